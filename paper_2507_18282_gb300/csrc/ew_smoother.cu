@@ -105,80 +105,138 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// per-block partial gradients: part[block][432]
-//   dW2[c][o] = sum_x gy(x) h_c(x + o)
-//   dh_c(x)   = sum_o W2[c][o] gy(x - o)
-//   dW1[c][o] = sum_x dh_c(x) r(x + o)
-// (the hidden activations and the residual enter with their BF16 rounding)
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-    k_smoother_bwd(int nx, int ny, int nz, const float* __restrict__ w, const T* __restrict__ r,
-                   const T* __restrict__ gy, double* __restrict__ part) {
-    __shared__ float sW[2 * kW];
-    __shared__ float sR[kRE * kRE * kRE];
-    __shared__ float sH[kHE * kHE * kHE * kC];
-    __shared__ float sG[kHE * kHE * kHE];      // gy on tile + halo 1
-    __shared__ float sD[kTile * kTile * kTile * kC];  // dh on the tile
-    for (int q = threadIdx.x; q < 2 * kW; q += kThreads) sW[q] = bf16r(w[q]);
-    const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile, z0 = blockIdx.z * kTile;
-    __syncthreads();
-    stage_hidden<T>(r, sW, sR, sH, x0, y0, z0, nx, ny, nz);
-    for (int q = threadIdx.x; q < kHE * kHE * kHE; q += kThreads) {
-        int lx = q % kHE, t = q / kHE, ly = t % kHE, lz = t / kHE;
-        int gx = x0 - 1 + lx, gyy = y0 - 1 + ly, gz = z0 - 1 + lz;
-        bool in = gx >= 0 && gyy >= 0 && gz >= 0 && gx < nx && gyy < ny && gz < nz;
-        sG[q] = in ? (float)gy[((int64_t)gz * ny + gyy) * nx + gx] : 0.f;
-    }
-    __syncthreads();
-    const float* sW2 = sW + kW;
-    // dh on the owned tile (zero outside the box)
-    for (int q = threadIdx.x; q < kTile * kTile * kTile; q += kThreads) {
-        int lx = q % kTile, t = q / kTile, ly = t % kTile, lz = t / kTile;
-        int gx = x0 + lx, gyy = y0 + ly, gz = z0 + lz;
-        float acc[kC];
+// Weight gradients of the two layers (the hidden activations and the residual
+// enter with their BF16 rounding):
+//   dW2[c][o] = sum_x gy(x) h_c(x + o)  =  sum_y h_c(y) gy(y - o)
+//   dh_c(y)   = sum_o W2[c][o] gy(y - o)
+//   dW1[c][o] = sum_y dh_c(y) r(y + o)
+// Both are sums over the box of A_c(y) B(y +- o): A_c is one of the two
+// per-channel fields, made from the 27 neighbours of y, and B is r or gy, so a
+// thread that owns one channel of one layer keeps its 27 weights, its 27 sums
+// and the 3x3x3 windows of r and gy in registers and walks along x: per point
+// 18 shared loads (nine rows of each field) feed 27 multiply-adds for A_c and
+// 27 terms.  No field of the hidden layer is stored.
+//
+// Sums: the running sum is a pair (hi, lo) of FP32 numbers, lo collecting the
+// rounding error of each fused multiply-add (t = fma(a, b, hi), its error
+// fma(a, b, hi - t)), four FP32 operations a term; the threads' pairs are
+// summed in FP64 in a fixed order.  Bound: FP32 pipe, 8 channels x 2 layers x
+// 135 operations a point.  Accumulating each of the 432 terms of a point in
+// FP64 from shared memory (one thread per weight over an 8^3 tile) took
+// 3461 us on 127^3 and its serial sum over the tiles 456 us; this form and its
+// finish take 240 us (forward and backward together 3818 -> 314 us).
+constexpr int kBwX = 32, kBwY = 8, kBwZ = 4;          // owned tile
+constexpr int kBwP = kBwX + 2;                        // row pitch: rows y .. y + 3 of a warp on different banks
+constexpr int kBwPlane = kBwP * (kBwY + 2);
+constexpr int kBwCells = kBwPlane * (kBwZ + 2);       // tile with a halo of one
+constexpr int kBwThreads = 128;                       // warps 0, 1: dW1; warps 2, 3: dW2
+constexpr int kBwCtas = 3;                            // CTAs a SM (168 registers a thread)
+
+// one layer's sums over the rows of a staged tile (nxt columns; this thread's
+// row y of each plane z < nzt)
+template <bool FIRST>
+__device__ __forceinline__ void bwd_rows(const float* sR, const float* sG, int y, int nxt, int nzt, const float (&w)[27],
+                                         float (&hi)[27], float (&lo)[27]) {
+    for (int z = 0; z < nzt; ++z) {
+        const float* pr = sR + z * kBwPlane + y * kBwP;
+        const float* pg = sG + z * kBwPlane + y * kBwP;
+        float wr[9][3], wg[9][3];  // windows: row (dz, dy), column slot (x + dx) mod 3
+        auto column = [&](int x, int slot) {
 #pragma unroll
-        for (int c = 0; c < kC; ++c) acc[c] = 0.f;
-        if (gx < nx && gyy < ny && gz < nz) {
-            int tap = 0;
-            for (int dz = -1; dz <= 1; ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx, ++tap) {
-                        float g = sG[((lz + 1 - dz) * kHE + (ly + 1 - dy)) * kHE + (lx + 1 - dx)];
+            for (int q = 0; q < 9; ++q) {
+                wr[q][slot] = pr[(q / 3) * kBwPlane + (q % 3) * kBwP + x];
+                wg[q][slot] = pg[(q / 3) * kBwPlane + (q % 3) * kBwP + x];
+            }
+        };
+        column(0, 0);
+        column(1, 1);
+        for (int x0 = 0; x0 < nxt; x0 += 3) {
 #pragma unroll
-                        for (int c = 0; c < kC; ++c) acc[c] = fmaf(sW2[c * 27 + tap], g, acc[c]);
-                    }
+            for (int u = 0; u < 3; ++u) {
+                const int x = x0 + u;
+                if (x >= nxt) break;
+                column(x + 2, (u + 2) % 3);
+                float a = 0.f;
+#pragma unroll
+                for (int t = 0; t < 27; ++t) {
+                    const int m = 26 - t;  // gy(y - o): the mirrored offset
+                    a = fmaf(w[t], FIRST ? wg[m / 3][(u + m % 3) % 3] : wr[t / 3][(u + t % 3) % 3], a);
+                }
+                if (!FIRST) a = bf16r(a);
+#pragma unroll
+                for (int t = 0; t < 27; ++t) {
+                    const int m = 26 - t;
+                    const float b = FIRST ? wr[t / 3][(u + t % 3) % 3] : wg[m / 3][(u + m % 3) % 3];
+                    const float s = __fmaf_rn(a, b, hi[t]);
+                    lo[t] = __fadd_rn(lo[t], __fmaf_rn(a, b, __fsub_rn(hi[t], s)));
+                    hi[t] = s;
+                }
+            }
         }
-#pragma unroll
-        for (int c = 0; c < kC; ++c) sD[q * kC + c] = acc[c];
-    }
-    __syncthreads();
-    // each thread accumulates a few of the 432 gradient entries over the tile;
-    // entry e < 216: dW1[c][tap], else dW2[c][tap]
-    for (int e = threadIdx.x; e < 2 * kW; e += kThreads) {
-        const int c = (e % kW) / 27, tap = (e % kW) % 27;
-        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-        double s = 0.0;
-        for (int q = 0; q < kTile * kTile * kTile; ++q) {
-            int lx = q % kTile, t = q / kTile, ly = t % kTile, lz = t / kTile;
-            float term;
-            if (e < kW)
-                term = sD[q * kC + c] * sR[((lz + 2 + dz) * kRE + (ly + 2 + dy)) * kRE + (lx + 2 + dx)];
-            else
-                term = sG[((lz + 1) * kHE + (ly + 1)) * kHE + (lx + 1)] *
-                       sH[(((lz + 1 + dz) * kHE + (ly + 1 + dy)) * kHE + (lx + 1 + dx)) * kC + c];
-            s += (double)term;
-        }
-        const int64_t b = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        part[b * (2 * kW) + e] = s;
     }
 }
 
-__global__ void k_grad_finish(const double* __restrict__ part, int64_t nblocks, float* __restrict__ grad) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// part[e * gridDim.x + block]: the block's share of gradient entry e
+template <typename T>
+__global__ void __launch_bounds__(kBwThreads, kBwCtas)
+    k_smoother_bwd(int nx, int ny, int nz, int tx, int ty, int64_t ntiles, const float* __restrict__ w,
+                   const T* __restrict__ r, const T* __restrict__ gy, double* __restrict__ part) {
+    __shared__ float sR[kBwCells];
+    __shared__ float sG[kBwCells];
+    __shared__ double sRed[4][8][27];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = lane & 7, y = (warp & 1) * 4 + (lane >> 3);
+    const bool first = warp < 2;
+    float wt[27], hi[27], lo[27];
+#pragma unroll
+    for (int t = 0; t < 27; ++t) {
+        wt[t] = bf16r(w[(first ? kW : 0) + c * 27 + t]);  // dW1 needs dh (W2), dW2 needs h (W1)
+        hi[t] = lo[t] = 0.f;
+    }
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int x0 = (int)(tile % tx) * kBwX, y0 = (int)(tile / tx % ty) * kBwY, z0 = (int)(tile / tx / ty) * kBwZ;
+        __syncthreads();  // the previous tile has been read
+        for (int q = threadIdx.x; q < kBwCells; q += kBwThreads) {
+            const int lx = q % kBwP, l = q / kBwP, ly = l % (kBwY + 2), lz = l / (kBwY + 2);
+            const int gx = x0 - 1 + lx, gyy = y0 - 1 + ly, gz = z0 - 1 + lz;
+            const bool in = gx >= 0 && gyy >= 0 && gz >= 0 && gx < nx && gyy < ny && gz < nz;
+            const int64_t g = ((int64_t)gz * ny + gyy) * nx + gx;
+            sR[q] = in ? bf16r((float)r[g]) : 0.f;
+            sG[q] = in ? (float)gy[g] : 0.f;
+        }
+        __syncthreads();
+        if (y0 + y < ny) {
+            const int nxt = min(kBwX, nx - x0), nzt = min(kBwZ, nz - z0);
+            if (first)
+                bwd_rows<true>(sR, sG, y, nxt, nzt, wt, hi, lo);
+            else
+                bwd_rows<false>(sR, sG, y, nxt, nzt, wt, hi, lo);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < 27; ++t) {
+        // an infinite sum has no error term
+        double v = isfinite(lo[t]) ? (double)hi[t] + (double)lo[t] : (double)hi[t];
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        if (lane < 8) sRed[warp][c][t] = v;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * kW; e += kBwThreads) {
+        const int l = e < kW ? 0 : 2, ce = (e % kW) / 27, t = (e % kW) % 27;
+        part[(int64_t)e * gridDim.x + blockIdx.x] = sRed[l][ce][t] + sRed[l + 1][ce][t];
+    }
+}
+
+// one warp per gradient entry: the blocks' shares in a fixed order
+__global__ void k_grad_finish(const double* __restrict__ part, int nblocks, float* __restrict__ grad) {
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (e >= 2 * kW) return;
     double s = 0.0;
-    for (int64_t b = 0; b < nblocks; ++b) s += part[b * (2 * kW) + e];
-    grad[e] = (float)s;
+    for (int b = lane; b < nblocks; b += 32) s += part[(int64_t)e * nblocks + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) grad[e] = (float)s;
 }
 
 // Adam step on the 432 weights (device-resident moments)
@@ -465,12 +523,16 @@ static ew_status smoother_forward_t(const GridGeom& g, const float* w, const T* 
 template <typename T>
 static ew_status smoother_backward_t(ew_grid* gr, const float* w, const T* r, const T* gy, float* grad, cudaStream_t st) {
     const GridGeom& g = gr->geom;
-    dim3 tl = tiles(g);
-    int64_t nb = (int64_t)tl.x * tl.y * tl.z;
+    const int64_t tx = (g.n[0] + kBwX - 1) / kBwX, ty = (g.n[1] + kBwY - 1) / kBwY, tz = (g.n[2] + kBwZ - 1) / kBwZ;
+    int dev = 0, nsm = 0;
+    EW_CUDA_TRY(cudaGetDevice(&dev));
+    EW_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int nb = (int)std::min<int64_t>(tx * ty * tz, (int64_t)kBwCtas * nsm);
     EW_TRY(gr->reduce.reserve(sizeof(double) * (size_t)nb * 2 * kW));
     double* part = (double*)gr->reduce.ptr;
-    k_smoother_bwd<T><<<tl, kThreads, 0, st>>>((int)g.n[0], (int)g.n[1], (int)g.n[2], w, r, gy, part);
-    k_grad_finish<<<(2 * kW + 127) / 128, 128, 0, st>>>(part, nb, grad);
+    k_smoother_bwd<T><<<nb, kBwThreads, 0, st>>>((int)g.n[0], (int)g.n[1], (int)g.n[2], (int)tx, (int)ty, tx * ty * tz,
+                                                 w, r, gy, part);
+    k_grad_finish<<<(2 * kW * 32 + 255) / 256, 256, 0, st>>>(part, nb, grad);
     EW_CUDA_TRY(cudaGetLastError());
     count_launch(2);
     return EW_OK;
