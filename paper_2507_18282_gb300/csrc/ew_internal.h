@@ -256,6 +256,13 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
                               const T* vin, T* vout, int nvec, T* fields, int temporal_block,
                               cudaStream_t st);
 
+// --- whole wave-solve of a small 2D grid on chip (ew_resident.cu) ------------
+template <typename T>
+bool resident_fits(const GridGeom& g, int nvec);
+template <typename T>
+ew_status resident_wave_solve(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
+                              cudaStream_t st);
+
 // --- curvilinear grids (ew_mapped.cu) ----------------------------------------
 ew_status mapped_build(int64_t n1, int64_t n2, const double* xy, MappedData* m);
 void mapped_release(MappedData* m);

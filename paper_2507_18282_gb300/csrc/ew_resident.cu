@@ -1,0 +1,439 @@
+// ew_resident.cu -- the whole explicit wave-solve of a small 2D grid on chip:
+// the grid and its ghost layers stay in shared memory (of one CTA, or of a
+// cluster of CTAs that exchange their edge rows through distributed shared
+// memory), D^n and the filter sums beside them, for all N_t steps of one
+// launch (eqs. explicitStep1, explicitScheme, filterQuadrature; the summed
+// form of ew_stencil.cu).
+#include <cooperative_groups.h>
+#include <stdlib.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "ew_bc_dev.cuh"
+#include "ew_dd.cuh"
+#include "ew_internal.h"
+
+namespace ew {
+
+// ---------------------------------------------------------------------------
+// whole wave-solve of a small 2D grid in one CTA
+// ---------------------------------------------------------------------------
+// boundary and ghost layers of a whole padded 2D grid (pitch PX, G = 2
+// layers on every side) from the box closure: Dirichlet walls 0, beyond them
+// the odd reflection, Neumann ghosts the even reflection.  The cross-shaped
+// stencils never read the corner blocks.
+template <typename T, int R>
+__device__ __forceinline__ void resident_fix(T* buf, int nx, int ny, int PX, int bc, int tid, int nthr) {
+    constexpr int G = 2;
+    if (R != 2 && bc == 0) return;  // order 2 with Dirichlet walls reads only the zero wall layer
+    const int bx = axis_bc(bc, 0), by = axis_bc(bc, 1);
+    for (int q = tid; q < 2 * G * (ny + nx); q += nthr) {
+        const int layer = q % G + 1, side = (q / G) & 1, r = q / (2 * G);
+        int sg = 1;
+        if (r < ny) {  // x-ghost of row r
+            const int gx = side ? nx - 1 + layer : -layer;
+            const int ix = ext_axis<int>(gx, nx, bx, sg);
+            const T v = ix < 0 ? T(0) : buf[(r + G) * PX + ix + G];
+            buf[(r + G) * PX + gx + G] = sg < 0 ? -v : v;
+        } else {  // y-ghost of column x
+            const int x = r - ny;
+            const int gy = side ? ny - 1 + layer : -layer;
+            const int iy = ext_axis<int>(gy, ny, by, sg);
+            const T v = iy < 0 ? T(0) : buf[(iy + G) * PX + x + G];
+            buf[(gy + G) * PX + x + G] = sg < 0 ? -v : v;
+        }
+    }
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(1024)
+    k_resident2d(int nx, int ny, const T* __restrict__ vin, T* __restrict__ vout,
+                 const T* __restrict__ cw, int64_t Nt, Stencil<T> st, Stencil<T> st_half) {
+    constexpr int G = 2;
+    const int PX = nx + 2 * G, PY = ny + 2 * G;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* sA = reinterpret_cast<T*>(smem_raw);
+    T* sB = sA + PX * PY;
+    T* sAcc = sB + PX * PY;
+    const int64_t N = (int64_t)nx * ny;
+    vin += blockIdx.x * N;
+    vout += blockIdx.x * N;
+    const int nthr = blockDim.x;
+    const int tid = threadIdx.x;
+
+    auto fix = [&](T* buf) { resident_fix<T, R>(buf, nx, ny, PX, st.bc, tid, nthr); };
+    auto lap = [&](const T* c, int p, const Stencil<T>& s) {
+        T r = s.c0 * c[p] + s.c1[0] * (c[p - 1] + c[p + 1]) + s.c1[1] * (c[p - PX] + c[p + PX]);
+        if (R == 2) r += s.c2[0] * (c[p - 2] + c[p + 2]) + s.c2[1] * (c[p - 2 * PX] + c[p + 2 * PX]);
+        return r;
+    };
+
+    // sA: W^n with its boundary and ghost layers; sB: D^n (same layout)
+    for (int q = tid; q < PX * PY; q += nthr) {
+        sA[q] = T(0);
+        sB[q] = T(0);
+    }
+    __syncthreads();
+    for (int q = tid; q < N; q += nthr) {
+        int x = q % nx, y = q / nx;
+        sA[(y + G) * PX + x + G] = vin[q];
+    }
+    __syncthreads();
+    fix(sA);
+    __syncthreads();
+    // first step (eq. explicitStep1): D^1 = (dt^2/2) L W^0, then W^1 = W^0 + D^1
+    const T c0 = cw[0], c1 = cw[1];
+    for (int q = tid; q < N; q += nthr) {
+        int x = q % nx, y = q / nx;
+        int p = (y + G) * PX + x + G;
+        sB[p] = lap(sA, p, st_half);
+    }
+    __syncthreads();
+    for (int q = tid; q < N; q += nthr) {
+        int x = q % nx, y = q / nx;
+        int p = (y + G) * PX + x + G;
+        T x0 = sA[p];
+        T w1 = x0 + sB[p];
+        sA[p] = w1;
+        sAcc[q] = c0 * x0 + c1 * w1;
+    }
+    __syncthreads();
+    fix(sA);
+    __syncthreads();
+    for (int64_t n = 1; n < Nt; ++n) {
+        const T cn = cw[n + 1];
+        // D^{n+1} = D^n + dt^2 L W^n everywhere, then W^{n+1} = W^n + D^{n+1} pointwise
+        for (int q = tid; q < N; q += nthr) {
+            int x = q % nx, y = q / nx;
+            int p = (y + G) * PX + x + G;
+            sB[p] = sB[p] + lap(sA, p, st);
+        }
+        __syncthreads();
+        for (int q = tid; q < N; q += nthr) {
+            int x = q % nx, y = q / nx;
+            int p = (y + G) * PX + x + G;
+            T wn = sA[p] + sB[p];
+            sA[p] = wn;
+            sAcc[q] += cn * wn;
+        }
+        __syncthreads();
+        fix(sA);
+        __syncthreads();
+    }
+    for (int q = tid; q < N; q += nthr) vout[q] = sAcc[q];
+}
+
+// one operation each, rounded once (double-FP32 pairs: ew_dd.cuh)
+__device__ __forceinline__ float r_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float r_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float r_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double r_add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double r_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double r_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ dd r_add(dd a, dd b) { return dd_add(a, b); }
+__device__ __forceinline__ dd r_mul(dd a, dd b) { return dd_mul(a, b); }
+__device__ __forceinline__ dd r_fma(dd a, dd b, dd c) { return dd_fma(a, b, c); }
+
+// The same on a cluster of CTAs: the rows of one vector's grid are split over
+// the CTAs of a cluster (each on an SM of its own), W^n is double-buffered in
+// their shared memory and D^n, W^n and the filter sums of a thread's points
+// stay in its registers, so a step is one pass and one cluster barrier.  A
+// thread that writes W^{n+1} of a point also writes the copies others need of
+// it: into the halo rows of the CTA above or below (distributed shared
+// memory), and into the ghost layers beyond the box's faces.
+//
+// The update of a point takes the operations of the blocked 2D kernels in
+// their order (BLOCKED, grids that those kernels serve in other calls: the
+// same bits either way) or those of k_resident2d (the grids of one CTA).
+//
+// Why: one CTA is bound by the units of one SM (FP64: two operations a clock;
+// 63^2 took 11 us a step), and its step was three passes over shared memory
+// with two integer divisions a point; the blocked kernels' tiles are about
+// 120 x 60 points and more, so up to a few 10,000 points they leave most SMs
+// idle and pay a launch for a few steps.  Measured, order 2, 400 steps, one
+// vector: 63^2 FP64 4290 (one CTA) -> 490 us, 127^2 FP64 4935 (blocked) ->
+// 1319 us, 181^2 in pairs 2939 -> 855 us, 255^2 FP32 order 4 1340 -> 597 us.
+// Bound: below about 500 points a CTA the cluster barrier (0.5 us a step),
+// above it the FP64 units or the shared-memory reads of the point loop.
+template <typename T, int R, int PT, bool BLOCKED>
+__global__ void __launch_bounds__(1024)
+    k_resident2d_cluster(int nx, int ny, const T* __restrict__ vin, T* __restrict__ vout, const T* __restrict__ cw,
+                         int64_t Nt, Stencil<T> st, Stencil<T> st_half) {
+    constexpr int G = 2;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int base = ny / C, rem = ny % C;
+    const int rows = base + (rank < rem), y0 = rank * base + min(rank, rem);
+    const int PX = nx + 2 * G, plane = (base + (rem > 0) + 2 * G) * PX;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* own = reinterpret_cast<T*>(smem_raw);  // W^n and W^{n+1}: local row ly at row ly + G
+    T* prev = rank > 0 ? cluster.map_shared_rank(own, rank - 1) : own;
+    T* next = rank + 1 < C ? cluster.map_shared_rank(own, rank + 1) : own;
+    const int64_t N = (int64_t)nx * ny, v = blockIdx.x / C;
+    const int nthr = blockDim.x, tid = threadIdx.x, npt = rows * nx;
+    vin += v * N + (int64_t)y0 * nx;
+    vout += v * N + (int64_t)y0 * nx;
+    for (int q = tid; q < 2 * plane; q += nthr) own[q] = T(0);  // walls stay 0
+
+    // a thread's points: index in a buffer, and where copies of it go (-1: nowhere)
+    const int bx = axis_bc(st.bc, 0), by = axis_bc(st.bc, 1);
+    const bool xl_odd = !(bx & 1), xh_odd = !(bx & 2), yl_odd = !(by & 1), yh_odd = !(by & 2);
+    int p[PT], cxl[PT], cxh[PT], cyl[PT], cyh[PT];
+#pragma unroll
+    for (int k = 0; k < PT; ++k) {
+        const int q = tid + k * nthr, ly = q / nx, x = q - ly * nx;
+        p[k] = q < npt ? (ly + G) * PX + x + G : -1;
+        cxl[k] = cxh[k] = cyl[k] = cyh[k] = -1;
+        if (q >= npt) continue;
+        // distance of the ghost a point feeds beyond each face: odd reflection about the wall
+        // one step outside (only point 0, two steps out), even about the wall point itself
+        const int dxl = xl_odd ? (R == 2 && x == 0 ? 2 : 0) : (x <= R ? x : 0);
+        const int hx = nx - 1 - x, dxh = xh_odd ? (R == 2 && hx == 0 ? 2 : 0) : (hx <= R ? hx : 0);
+        if (dxl) cxl[k] = (ly + G) * PX + G - dxl;
+        if (dxh) cxh[k] = (ly + G) * PX + G + nx - 1 + dxh;
+        const int hy = rows - 1 - ly;
+        if (rank == 0) {
+            const int d = yl_odd ? (R == 2 && ly == 0 ? 2 : 0) : (ly <= R ? ly : 0);
+            if (d) cyl[k] = (G - d) * PX + x + G;
+        } else if (ly < R) {
+            cyl[k] = (base + (rank - 1 < rem) + G + ly) * PX + x + G;
+        }
+        if (rank == C - 1) {
+            const int d = yh_odd ? (R == 2 && hy == 0 ? 2 : 0) : (hy <= R ? hy : 0);
+            if (d) cyh[k] = (G + rows - 1 + d) * PX + x + G;
+        } else if (hy < R) {
+            cyh[k] = (G - 1 - hy) * PX + x + G;
+        }
+    }
+    const bool yl_neg = rank == 0 && yl_odd, yh_neg = rank == C - 1 && yh_odd;
+    auto put = [&](int off, int k, T w) {  // W of point k into buffer `off` and its copies
+        own[off + p[k]] = w;
+        if (cxl[k] >= 0) own[off + cxl[k]] = xl_odd ? -w : w;
+        if (cxh[k] >= 0) own[off + cxh[k]] = xh_odd ? -w : w;
+        if (cyl[k] >= 0) prev[off + cyl[k]] = yl_neg ? -w : w;
+        if (cyh[k] >= 0) next[off + cyh[k]] = yh_neg ? -w : w;
+    };
+    auto sync = [&]() {
+        if (C > 1)
+            cluster.sync();
+        else
+            __syncthreads();
+    };
+    auto lap = [&](const T* c, int q, T u, const Stencil<T>& s) {
+        if constexpr (BLOCKED) {
+            T r = r_mul(s.c0, u);
+            r = r_fma(s.c1[0], r_add(c[q - 1], c[q + 1]), r);
+            r = r_fma(s.c1[1], r_add(c[q - PX], c[q + PX]), r);
+            if (R == 2) {
+                r = r_fma(s.c2[0], r_add(c[q - 2], c[q + 2]), r);
+                r = r_fma(s.c2[1], r_add(c[q - 2 * PX], c[q + 2 * PX]), r);
+            }
+            return r;
+        }
+        T r = s.c0 * c[q] + s.c1[0] * (c[q - 1] + c[q + 1]) + s.c1[1] * (c[q - PX] + c[q + PX]);
+        if (R == 2) r += s.c2[0] * (c[q - 2] + c[q + 2]) + s.c2[1] * (c[q - 2 * PX] + c[q + 2 * PX]);
+        return r;
+    };
+    sync();
+    T w[PT], d[PT], acc[PT];
+#pragma unroll
+    for (int k = 0; k < PT; ++k) {
+        w[k] = d[k] = acc[k] = T(0);
+        if (p[k] >= 0) {
+            w[k] = vin[tid + k * nthr];
+            put(0, k, w[k]);
+        }
+    }
+    sync();
+    const T c0 = cw[0], c1 = cw[1];
+#pragma unroll
+    for (int k = 0; k < PT; ++k)
+        if (p[k] >= 0) {
+            if constexpr (BLOCKED) {  // the sum of k_first_step2d
+                T r = st_half.c0 * w[k];
+                r += st_half.c1[0] * (own[p[k] - 1] + own[p[k] + 1]);
+                r += st_half.c1[1] * (own[p[k] - PX] + own[p[k] + PX]);
+                if (R == 2) {
+                    r += st_half.c2[0] * (own[p[k] - 2] + own[p[k] + 2]);
+                    r += st_half.c2[1] * (own[p[k] - 2 * PX] + own[p[k] + 2 * PX]);
+                }
+                d[k] = r;
+            } else {
+                d[k] = lap(own, p[k], w[k], st_half);
+            }
+            const T w1 = w[k] + d[k];
+            acc[k] = c0 * w[k] + c1 * w1;
+            w[k] = w1;
+            put(plane, k, w1);
+        }
+    int cur = plane;
+    T cn = Nt > 1 ? cw[2] : T(0);
+    for (int64_t n = 1; n < Nt; ++n) {
+        sync();
+        const T cs = cn;
+        if (n + 1 < Nt) cn = cw[n + 2];
+        const int nxt = plane - cur;
+#pragma unroll
+        for (int k = 0; k < PT; ++k)
+            if (p[k] >= 0) {
+                T wn;
+                if constexpr (BLOCKED) {
+                    d[k] = r_add(d[k], lap(own + cur, p[k], w[k], st));
+                    wn = r_add(w[k], d[k]);
+                    acc[k] = r_fma(cs, wn, acc[k]);
+                } else {
+                    d[k] = d[k] + lap(own + cur, p[k], w[k], st);
+                    wn = w[k] + d[k];
+                    acc[k] += cs * wn;
+                }
+                w[k] = wn;
+                put(nxt, k, wn);
+            }
+        cur = nxt;
+    }
+    sync();  // no CTA leaves while another may still write into its shared memory
+#pragma unroll
+    for (int k = 0; k < PT; ++k)
+        if (p[k] >= 0) vout[tid + k * nthr] = acc[k];
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+template <typename T>
+static size_t resident_smem(const GridGeom& g) {
+    return sizeof(T) * ((size_t)2 * (g.n[0] + 4) * (g.n[1] + 4) + (size_t)g.n[0] * g.n[1]);
+}
+
+// one CTA a vector: every grid of up to 16384 points whose three fields fit its shared memory
+template <typename T>
+static bool fits_cta(const GridGeom& g, int nvec) {
+    return resident_smem<T>(g) <= 200 * 1024 && g.N <= 16384 && nvec <= 4 * 152;
+}
+
+constexpr int kResMaxPts = 4096;  // points a CTA of the cluster form (four a thread)
+
+// CTAs a cluster for nvec vectors of this grid; 0: not the cluster form.
+// Sixteen CTAs a vector are the fastest up to 16 vectors (63^2 and 127^2, all
+// types: e.g. 127^2 in FP64, 16 vectors, 3.55 ms against 4.79 ms with 8); with
+// more vectors the SMs fill anyway, so fewer CTAs a vector pay fewer barriers
+// (63^2 in FP32, 64 vectors: 194 us with 2, 309 us with 4).  Small grids take
+// one CTA where the barrier would cost more than it spreads: below about 2000
+// points in FP32 (31^2, 200 steps: 76 us against 128 us with 4), 900 in pairs,
+// 400 in FP64.
+template <typename T>
+static int cluster_ctas(const GridGeom& g, int nvec) {
+    if (g.n[0] < 4 || g.n[1] < 4) return 0;  // ghosts mirror points of the edge CTAs only
+    const int small = sizeof(T) == 4 ? 2048 : std::is_same<T, dd>::value ? 900 : 400;
+    int C = nvec <= 16 ? 16 : nvec <= 36 ? 4 : nvec <= 76 ? 2 : 1;
+    if (g.N < small) C = 1;
+    while (C > 1 && g.n[1] < 3 * C) C /= 2;
+    while (C < 16 && (g.n[1] + C - 1) / C * g.n[0] > kResMaxPts) C *= 2;
+    if (g.n[1] < 3 * C || (g.n[1] + C - 1) / C * g.n[0] > kResMaxPts) return 0;
+    // FP64 with one CTA a vector: the one-CTA form's passes are 8-20 % faster (31^2, 63^2, 256 vectors)
+    if (std::is_same<T, double>::value && C == 1) return 0;
+    return C;
+}
+
+// The cluster form also takes larger grids with few vectors, which the blocked
+// kernels would run on a fraction of the SMs.  The line is where both took the
+// same time (400 steps): FP32 up to 4 x 255^2 points (order 4: 656 against
+// 1354 us; 16 x 181^2 1199 against 1358 us is left to the blocked form's
+// larger tiles); pairs 16 x 255^2 (3838 against 5781 us); FP64 4 x 255^2
+// (4830 against 4938 us), and 16 x 127^2 (3554 against 8124 us).
+template <typename T>
+static bool fits_cluster(const GridGeom& g, int nvec) {
+    if (g.N > 65536 || !cluster_ctas<T>(g, nvec)) return false;
+    if (std::is_same<T, dd>::value) return nvec <= 16;
+    if (g.N * nvec > 262144 + 2048) return false;
+    return sizeof(T) == 4 || g.N <= 16384 || nvec <= 4;
+}
+
+template <typename T>
+bool resident_fits(const GridGeom& g, int nvec) {
+    return g.dim == 2 && !g.map && (fits_cta<T>(g, nvec) || fits_cluster<T>(g, nvec));
+}
+template bool resident_fits<float>(const GridGeom&, int);
+template bool resident_fits<double>(const GridGeom&, int);
+template bool resident_fits<dd>(const GridGeom&, int);
+
+// one-CTA form
+template <typename T, int R>
+static ew_status resident_cta(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
+                              const Stencil<T>& s, const Stencil<T>& sh, cudaStream_t st) {
+    const size_t smem = resident_smem<T>(g);
+    const int threads = (int)std::min<int64_t>(1024, ((g.N + 31) / 32) * 32);
+    EW_CUDA_TRY(cudaFuncSetAttribute(k_resident2d<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_resident2d<T, R><<<nvec, threads, smem, st>>>((int)g.n[0], (int)g.n[1], vin, vout, cw, plan.Nt, s, sh);
+    EW_CUDA_TRY(cudaGetLastError());
+    return EW_OK;
+}
+
+template <typename T, int R, int PT, bool BLOCKED>
+static ew_status resident_cluster_pt(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan,
+                                     int nvec, int C, int threads, const Stencil<T>& s, const Stencil<T>& sh,
+                                     cudaStream_t st) {
+    const size_t smem = 2 * sizeof(T) * (size_t)((g.n[1] + C - 1) / C + 4) * (size_t)(g.n[0] + 4);
+    auto kern = k_resident2d_cluster<T, R, PT, BLOCKED>;
+    EW_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    EW_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nvec * C));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    EW_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (int)g.n[0], (int)g.n[1], vin, vout, cw, plan.Nt, s, sh));
+    return EW_OK;
+}
+
+template <typename T, int R, bool BLOCKED>
+static ew_status resident_cluster(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan,
+                                  int nvec, int C, const Stencil<T>& s, const Stencil<T>& sh, cudaStream_t st) {
+    // points a thread: 512 threads beat 1024 once each has two points (a barrier of fewer warps;
+    // 127^2 FP32 order 4, 16 CTAs, 8 vectors, 400 steps: 565 us with one point, 365 with two, 408 with four)
+    const int64_t pts = (g.n[1] + C - 1) / C * g.n[0];  // points of the fullest CTA
+    const int PT = pts <= 512 ? 1 : pts <= 1024 ? 2 : 4;
+    const int threads = (int)(((pts + PT - 1) / PT + 31) / 32 * 32);
+    if (PT == 1) return resident_cluster_pt<T, R, 1, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
+    if (PT == 2) return resident_cluster_pt<T, R, 2, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
+    return resident_cluster_pt<T, R, 4, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
+}
+
+template <typename T, int R>
+static ew_status resident_r(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
+                            cudaStream_t st) {
+    const Stencil<T> s = make_stencil<T>(g, plan.dt * plan.dt);
+    const Stencil<T> sh = make_stencil<T>(g, 0.5 * plan.dt * plan.dt);
+    const int C = cluster_ctas<T>(g, nvec);
+    if (!fits_cta<T>(g, nvec)) return resident_cluster<T, R, true>(g, vin, vout, cw, plan, nvec, C, s, sh, st);
+    if (C > 0) return resident_cluster<T, R, false>(g, vin, vout, cw, plan, nvec, C, s, sh, st);
+    return resident_cta<T, R>(g, vin, vout, cw, plan, nvec, s, sh, st);
+}
+
+template <typename T>
+ew_status resident_wave_solve(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
+                              cudaStream_t st) {
+    cudaEvent_t ev = fused_begin(st);
+    if (g.order == 2)
+        EW_TRY((resident_r<T, 1>(g, vin, vout, cw, plan, nvec, st)));
+    else
+        EW_TRY((resident_r<T, 2>(g, vin, vout, cw, plan, nvec, st)));
+    fused_end(ev, st, g.N * nvec, g.N * nvec * plan.Nt);
+    return EW_OK;
+}
+template ew_status resident_wave_solve<float>(const GridGeom&, const float*, float*, const float*, const FilterPlan&,
+                                              int, cudaStream_t);
+template ew_status resident_wave_solve<double>(const GridGeom&, const double*, double*, const double*,
+                                               const FilterPlan&, int, cudaStream_t);
+template ew_status resident_wave_solve<dd>(const GridGeom&, const dd*, dd*, const dd*, const FilterPlan&, int,
+                                           cudaStream_t);
+
+}  // namespace ew

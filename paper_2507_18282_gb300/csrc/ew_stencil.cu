@@ -34,8 +34,8 @@
 //                       V_out += c W^{n+1}.
 //   k_step_tb2d       : (ew_tb2d.cu) b time steps per launch on overlapped
 //                       tiles staged in shared memory (temporal blocking).
-//   k_resident2d      : the whole wave-solve of a small 2D grid inside one CTA
-//                       (grid + ghosts resident in shared memory).
+//   k_resident2d*     : (ew_resident.cu) the whole wave-solve of a small 2D grid
+//                       on chip, in one CTA or a cluster of them.
 #include <algorithm>
 #include <cmath>
 #include <limits>
@@ -219,114 +219,6 @@ __global__ void k_step_simple(int64_t nx, int64_t ny, int64_t nz, const T* __res
 }
 
 // ---------------------------------------------------------------------------
-// whole wave-solve of a small 2D grid in one CTA
-// ---------------------------------------------------------------------------
-// boundary and ghost layers of a whole padded 2D grid (pitch PX, G = 2
-// layers on every side) from the box closure: Dirichlet walls 0, beyond them
-// the odd reflection, Neumann ghosts the even reflection.  The cross-shaped
-// stencils never read the corner blocks.
-template <typename T, int R>
-__device__ __forceinline__ void resident_fix(T* buf, int nx, int ny, int PX, int bc, int tid, int nthr) {
-    constexpr int G = 2;
-    if (R != 2 && bc == 0) return;  // order 2 with Dirichlet walls reads only the zero wall layer
-    const int bx = axis_bc(bc, 0), by = axis_bc(bc, 1);
-    for (int q = tid; q < 2 * G * (ny + nx); q += nthr) {
-        const int layer = q % G + 1, side = (q / G) & 1, r = q / (2 * G);
-        int sg = 1;
-        if (r < ny) {  // x-ghost of row r
-            const int gx = side ? nx - 1 + layer : -layer;
-            const int ix = ext_axis<int>(gx, nx, bx, sg);
-            const T v = ix < 0 ? T(0) : buf[(r + G) * PX + ix + G];
-            buf[(r + G) * PX + gx + G] = sg < 0 ? -v : v;
-        } else {  // y-ghost of column x
-            const int x = r - ny;
-            const int gy = side ? ny - 1 + layer : -layer;
-            const int iy = ext_axis<int>(gy, ny, by, sg);
-            const T v = iy < 0 ? T(0) : buf[(iy + G) * PX + x + G];
-            buf[(gy + G) * PX + x + G] = sg < 0 ? -v : v;
-        }
-    }
-}
-
-template <typename T, int R>
-__global__ void __launch_bounds__(1024)
-    k_resident2d(int nx, int ny, const T* __restrict__ vin, T* __restrict__ vout,
-                 const T* __restrict__ cw, int64_t Nt, Stencil<T> st, Stencil<T> st_half) {
-    constexpr int G = 2;
-    const int PX = nx + 2 * G, PY = ny + 2 * G;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sA = reinterpret_cast<T*>(smem_raw);
-    T* sB = sA + PX * PY;
-    T* sAcc = sB + PX * PY;
-    const int64_t N = (int64_t)nx * ny;
-    vin += blockIdx.x * N;
-    vout += blockIdx.x * N;
-    const int nthr = blockDim.x;
-    const int tid = threadIdx.x;
-
-    auto fix = [&](T* buf) { resident_fix<T, R>(buf, nx, ny, PX, st.bc, tid, nthr); };
-    auto lap = [&](const T* c, int p, const Stencil<T>& s) {
-        T r = s.c0 * c[p] + s.c1[0] * (c[p - 1] + c[p + 1]) + s.c1[1] * (c[p - PX] + c[p + PX]);
-        if (R == 2) r += s.c2[0] * (c[p - 2] + c[p + 2]) + s.c2[1] * (c[p - 2 * PX] + c[p + 2 * PX]);
-        return r;
-    };
-
-    // sA: W^n with its boundary and ghost layers; sB: D^n (same layout)
-    for (int q = tid; q < PX * PY; q += nthr) {
-        sA[q] = T(0);
-        sB[q] = T(0);
-    }
-    __syncthreads();
-    for (int q = tid; q < N; q += nthr) {
-        int x = q % nx, y = q / nx;
-        sA[(y + G) * PX + x + G] = vin[q];
-    }
-    __syncthreads();
-    fix(sA);
-    __syncthreads();
-    // first step (eq. explicitStep1): D^1 = (dt^2/2) L W^0, then W^1 = W^0 + D^1
-    const T c0 = cw[0], c1 = cw[1];
-    for (int q = tid; q < N; q += nthr) {
-        int x = q % nx, y = q / nx;
-        int p = (y + G) * PX + x + G;
-        sB[p] = lap(sA, p, st_half);
-    }
-    __syncthreads();
-    for (int q = tid; q < N; q += nthr) {
-        int x = q % nx, y = q / nx;
-        int p = (y + G) * PX + x + G;
-        T x0 = sA[p];
-        T w1 = x0 + sB[p];
-        sA[p] = w1;
-        sAcc[q] = c0 * x0 + c1 * w1;
-    }
-    __syncthreads();
-    fix(sA);
-    __syncthreads();
-    for (int64_t n = 1; n < Nt; ++n) {
-        const T cn = cw[n + 1];
-        // D^{n+1} = D^n + dt^2 L W^n everywhere, then W^{n+1} = W^n + D^{n+1} pointwise
-        for (int q = tid; q < N; q += nthr) {
-            int x = q % nx, y = q / nx;
-            int p = (y + G) * PX + x + G;
-            sB[p] = sB[p] + lap(sA, p, st);
-        }
-        __syncthreads();
-        for (int q = tid; q < N; q += nthr) {
-            int x = q % nx, y = q / nx;
-            int p = (y + G) * PX + x + G;
-            T wn = sA[p] + sB[p];
-            sA[p] = wn;
-            sAcc[q] += cn * wn;
-        }
-        __syncthreads();
-        fix(sA);
-        __syncthreads();
-    }
-    for (int q = tid; q < N; q += nthr) vout[q] = sAcc[q];
-}
-
-// ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 // one thread per point: x from the block's threads, y from grid.y, z and the
@@ -369,11 +261,6 @@ template ew_status launch_apply_L<float>(const GridGeom&, const float*, float*, 
                                          cudaStream_t);
 template ew_status launch_apply_L<double>(const GridGeom&, const double*, double*, int, double,
                                           cudaStream_t);
-
-template <typename T>
-static size_t resident_smem(const GridGeom& g) {
-    return sizeof(T) * ((size_t)2 * (g.n[0] + 4) * (g.n[1] + 4) + (size_t)g.n[0] * g.n[1]);
-}
 
 template <typename T>
 ew_status step3d(const GridGeom& g, const T* W, T* D, T* Wout, T* acc, T c, const Stencil<T>& s, int nvec,
@@ -425,35 +312,6 @@ static ew_status step_simple(const GridGeom& g, const T* W, T* D, T* Wout, T* ac
 }
 
 template <typename T>
-static ew_status resident(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan,
-                          int nvec, cudaStream_t st) {
-    Stencil<T> s = make_stencil<T>(g, plan.dt * plan.dt);
-    Stencil<T> sh = make_stencil<T>(g, 0.5 * plan.dt * plan.dt);
-    size_t smem = resident_smem<T>(g);
-    int threads = (int)std::min<int64_t>(1024, ((g.N + 31) / 32) * 32);
-    cudaEvent_t ev = fused_begin(st);
-    if (g.order == 2) {
-        EW_CUDA_TRY(cudaFuncSetAttribute(k_resident2d<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-        k_resident2d<T, 1><<<nvec, threads, smem, st>>>((int)g.n[0], (int)g.n[1], vin, vout, cw, plan.Nt, s, sh);
-    } else {
-        EW_CUDA_TRY(cudaFuncSetAttribute(k_resident2d<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-        k_resident2d<T, 2><<<nvec, threads, smem, st>>>((int)g.n[0], (int)g.n[1], vin, vout, cw, plan.Nt, s, sh);
-    }
-    EW_CUDA_TRY(cudaGetLastError());
-    fused_end(ev, st, g.N * nvec, g.N * nvec * plan.Nt);
-    return EW_OK;
-}
-
-// Resident path: small 2D grids whose three fields fit in one CTA's shared
-// memory and would leave most SMs idle anyway.
-template <typename T>
-static bool use_resident(const GridGeom& g, int nvec) {
-    return g.dim == 2 && resident_smem<T>(g) <= 200 * 1024 && g.N <= 16384 && nvec <= 4 * 152;
-}
-
-template <typename T>
 ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* cdev, const T* vin, T* vout,
                               int nvec, T* fields, int temporal_block, cudaStream_t st) {
     if (temporal_block < 0) return set_error(EW_EINVAL, "temporal_block < 0");
@@ -464,9 +322,9 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
         if (g.map) return mapped_wave_solve<T>(g, plan, vin, vout, nvec, fields, st);  // one step per launch
     }
     // the variant override EW_TB2D_VARIANT (a tuning and testing hook) selects a
-    // blocked kernel, so it also bypasses the one-CTA path of small grids
-    if (use_resident<T>(g, nvec) && temporal_block == 0 && !getenv("EW_TB2D_VARIANT"))
-        return resident<T>(g, vin, vout, cdev, plan, nvec, st);
+    // blocked kernel, so it also bypasses the on-chip path of small grids
+    if (temporal_block == 0 && resident_fits<T>(g, nvec) && !getenv("EW_TB2D_VARIANT"))
+        return resident_wave_solve<T>(g, vin, vout, cdev, plan, nvec, st);
     // fields are laid out [field][vector][point]; 2D rows may be padded (pitch2d)
     const int64_t fstride = wave_field_stride(g);
     T* F[4];
