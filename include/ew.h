@@ -121,7 +121,7 @@ void ew_grid_destroy(ew_grid* grid);
  * in those weights).  The explicit step limit comes from a Gershgorin bound
  * of rho(-L).  EW_EINVAL if J <= 0 at some vertex.  Like ew_grid_create it
  * needs no GPU; the couplings are copied to the device on first use.
- * ew_filter_apply (explicit scheme, one step per launch; temporal_block is
+ * ew_filter_apply (explicit scheme; temporal_block is
  * ignored), ew_filter_apply_batched, ew_apply_L, ew_rayleigh,
  * ew_power_iteration and ew_arnoldi_eigs accept such grids; the implicit
  * scheme, multigrid, ew_filter_apply_noalloc and ew_choose_num_periods return

@@ -496,6 +496,7 @@ static ew_status rayleigh_t(ew_grid* g, const T* phi, int nvec, double* lam_host
     EW_CUDA_TRY(cudaStreamSynchronize(st));
     EW_TRY(rb2d_check_timeout());  // a register-blocked wave-solve before this point gave up a wait
     EW_TRY(tma2d_check_timeout());  // the same for a TMA-staged one
+    if (g->geom.map) EW_TRY(mapped_check_timeout());
     std::vector<double> lam2(nvec);
     for (int j = 0; j < nvec; ++j) {
         double den = h[nvec + j];

@@ -122,7 +122,7 @@ struct MappedData {
     std::vector<double> J;
     std::vector<double> xy;
     double rho = 0.0;
-    void* dev[2] = {nullptr, nullptr};  // per vertex (E, N, NE, SE), then (centre, 1/J): FP32 / FP64
+    void* dev[2] = {nullptr, nullptr};  // planes E, N, NE, SE, centre, 1/J of padded row pitch: FP32 / FP64
     double* sqrtJ = nullptr;
     std::mutex mu;
 };
@@ -269,8 +269,14 @@ void mapped_release(MappedData* m);
 template <typename T>
 ew_status mapped_apply_L(const GridGeom& g, const T* u, T* Lu, int nvec, double scale, cudaStream_t st);
 template <typename T>
-ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* vin, T* vout, int nvec, T* fields,
-                            cudaStream_t st);
+ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* cdev, const T* vin, T* vout, int nvec,
+                            T* fields, cudaStream_t st);
+// temporally blocked FP32 steps 2 .. N_t (ew_mapped_tb.cu): F[0] = D^1, F[1] = W^1 of padded row pitch,
+// c the six coupling planes; accumulates into acc
+ew_status mapped_advance(const GridGeom& g, const FilterPlan& plan, const float* c, const float* cdev, float* const* F,
+                         float* acc, int nvec, int64_t fstride, float dt2, cudaStream_t st);
+// reads (and clears) the flag a staging wait of the blocked curvilinear step sets when it gives up
+ew_status mapped_check_timeout();
 template <typename T>
 ew_status mapped_wsqrt(const GridGeom& g, const T* in, T* out, int nvec, int e, cudaStream_t st);
 

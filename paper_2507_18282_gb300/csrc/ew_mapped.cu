@@ -16,8 +16,8 @@
 // coupling of a vertex to its east neighbour equals the east neighbour's
 // coupling back, and likewise north, north-east and south-east.  So per
 // active vertex the library stores the centre and the E, N, NE, SE couplings
-// of J L (the W, S, SW, NW ones are the neighbours' E, N, NE, SE) and 1/J, as
-// one 4-wide record (E, N, NE, SE) and one 2-wide record (centre, 1/J) per vertex.
+// of J L (the W, S, SW, NW ones are the neighbours' E, N, NE, SE) and 1/J, in six
+// planes of padded row pitch (the TMA loads of ew_mapped_tb.cu).
 // The off-diagonal couplings are rounded to a common grid and the centre is
 // minus their exact sum, so L 1 = 0 holds exactly in the stored precision
 // (the same consistency as the box stencils).
@@ -26,11 +26,9 @@
 // product of the map), which ew_rayleigh and the Krylov solver use through the
 // weights sqrt(J) (launch_wsqrt).
 //
-// Kernels: one fused leapfrog + filter step per launch (summed form, as the
-// box kernels), the first step, and L alone.  Per point and step the step kernel
-// moves W^n, D^n and the filter sum in, the five couplings and 1/J in, and
-// D^{n+1}, W^{n+1} and the filter sum out: 48 B in FP32 (the neighbours' W and
-// couplings come through L1/L2).
+// Kernels: the first step, L alone, and one fused leapfrog + filter step per
+// launch (summed form, as the box kernels) for FP64, whose steps are bound by
+// the FP64 units; FP32 grids take several steps a launch (ew_mapped_tb.cu).
 #include <math.h>
 
 #include <algorithm>
@@ -127,7 +125,7 @@ ew_status mapped_build(int64_t n1, int64_t n2, const double* xy, MappedData* m) 
 // centre minus their exact sum (L 1 = 0 exactly in T)
 template <typename T>
 static void mapped_round(const MappedData& m, std::vector<T>& out) {
-    const int64_t n1 = m.n1, n2 = m.n2, p1 = n1 + 2, N = n1 * n2;
+    const int64_t n1 = m.n1, n2 = m.n2, p1 = n1 + 2;
     double mx = 0.0;
     for (size_t q = 0; q < m.E.size(); ++q)
         mx = std::max(std::max(mx, fabs(m.E[q])), std::max(fabs(m.N[q]), std::max(fabs(m.NE[q]), fabs(m.SE[q]))));
@@ -136,25 +134,23 @@ static void mapped_round(const MappedData& m, std::vector<T>& out) {
     frexp(16.0 * mx, &e);
     double q2 = 0.5 * ldexp(1.0, e - mant);
     auto rnd = [&](double c) { return nearbyint(c / q2) * q2; };
-    // layout: N records (E, N, NE, SE) then N records (centre, 1/J), so a point's
-    // own couplings are one 4-wide and one 2-wide load
-    out.assign((size_t)(6 * N), T(0));
-    T* quad = out.data();
-    T* pair = quad + 4 * N;
+    // layout: six planes E, N, NE, SE, centre, 1/J of n2 rows of pitch pitch2d(n1), zeros in the pad columns
+    const int64_t pitch = pitch2d(n1), plane = pitch * n2;
+    out.assign((size_t)(6 * plane), T(0));
     auto c = [&](const std::vector<double>& a, int64_t i, int64_t j) { return rnd(a[(size_t)(j * p1 + i)]); };
     for (int64_t J = 1; J <= n2; ++J)
         for (int64_t I = 1; I <= n1; ++I) {
-            const size_t q = (size_t)((J - 1) * n1 + (I - 1));
+            T* o = out.data() + (size_t)((J - 1) * pitch + (I - 1));
             const double off[8] = {c(m.E, I, J),     c(m.E, I - 1, J),      c(m.N, I, J),  c(m.N, I, J - 1),
                                    c(m.NE, I, J),    c(m.NE, I - 1, J - 1), c(m.SE, I, J), c(m.SE, I - 1, J + 1)};
             double centre = 0.0;
             for (double o : off) centre -= o;  // exact: multiples of q/2 far below 2^53 q/2
-            quad[4 * q + 0] = T(off[0]);
-            quad[4 * q + 1] = T(off[2]);
-            quad[4 * q + 2] = T(off[4]);
-            quad[4 * q + 3] = T(off[6]);
-            pair[2 * q + 0] = T(centre);
-            pair[2 * q + 1] = T(1.0 / m.J[q]);
+            o[0 * plane] = T(off[0]);
+            o[1 * plane] = T(off[2]);
+            o[2 * plane] = T(off[4]);
+            o[3 * plane] = T(off[6]);
+            o[4 * plane] = T(centre);
+            o[5 * plane] = T(1.0 / m.J[(size_t)((J - 1) * n1 + (I - 1))]);
         }
 }
 
@@ -205,71 +201,58 @@ void mapped_release(MappedData* m) {
     m->sqrtJ = nullptr;
 }
 
-// a point's own couplings: (E, N, NE, SE) and (centre, 1/J)
-template <typename T>
-struct Own {
-    T e, n, ne, se, c, rj;
-};
-__device__ __forceinline__ Own<float> own_couplings(const float* __restrict__ c, int64_t N, int64_t q) {
-    const float4 a = reinterpret_cast<const float4*>(c)[q];
-    const float2 b = reinterpret_cast<const float2*>(c + 4 * N)[q];
-    return Own<float>{a.x, a.y, a.z, a.w, b.x, b.y};
-}
-__device__ __forceinline__ Own<double> own_couplings(const double* __restrict__ c, int64_t N, int64_t q) {
-    const double2 a = reinterpret_cast<const double2*>(c)[2 * q];
-    const double2 a2 = reinterpret_cast<const double2*>(c)[2 * q + 1];
-    const double2 b = reinterpret_cast<const double2*>(c + 4 * N)[q];
-    return Own<double>{a.x, a.y, a2.x, a2.y, b.x, b.y};
-}
-
 // J L u at active vertex (i, j) (0-based), x fastest, and 1/J there; neighbours
-// beyond the active set are boundary vertices (u = 0)
+// beyond the active set are boundary vertices (u = 0).  c: the six coupling
+// planes, `plane` elements each, row pitch `pitch`
 template <typename T>
-__device__ __forceinline__ T mapped_jlap(const T* __restrict__ u, const T* __restrict__ c, int64_t N, int nx,
-                                         int ny, int i, int j, int64_t q, T& rj) {
-    const Own<T> o = own_couplings(c, N, q);
-    rj = o.rj;
+__device__ __forceinline__ T mapped_jlap(const T* __restrict__ u, const T* __restrict__ c, int pitch, int64_t plane,
+                                         int nx, int ny, int i, int j, int64_t q, T& rj) {
+    const int64_t p = (int64_t)j * pitch + i;
+    const T *cE = c + p, *cN = cE + plane, *cNE = cN + plane, *cSE = cNE + plane, *cC = cSE + plane;
+    rj = cC[plane];
     const bool w = i > 0, e = i + 1 < nx, s = j > 0, n = j + 1 < ny;
-    T r = o.c * u[q];
-    if (e) r += o.e * u[q + 1];
-    if (w) r += c[4 * (q - 1) + 0] * u[q - 1];
-    if (n) r += o.n * u[q + nx];
-    if (s) r += c[4 * (q - nx) + 1] * u[q - nx];
-    if (e && n) r += o.ne * u[q + 1 + nx];
-    if (w && s) r += c[4 * (q - 1 - nx) + 2] * u[q - 1 - nx];
-    if (e && s) r += o.se * u[q + 1 - nx];
-    if (w && n) r += c[4 * (q - 1 + nx) + 3] * u[q - 1 + nx];
+    T r = cC[0] * u[q];
+    if (e) r += cE[0] * u[q + 1];
+    if (w) r += cE[-1] * u[q - 1];
+    if (n) r += cN[0] * u[q + nx];
+    if (s) r += cN[-pitch] * u[q - nx];
+    if (e && n) r += cNE[0] * u[q + 1 + nx];
+    if (w && s) r += cNE[-1 - pitch] * u[q - 1 - nx];
+    if (e && s) r += cSE[0] * u[q + 1 - nx];
+    if (w && n) r += cSE[-1 + pitch] * u[q - 1 + nx];
     return r;
 }
 
 // one thread per point: x from the block's threads, y from grid.y, the vector from grid.z
 template <typename T>
 __global__ void __launch_bounds__(128) k_mapped_apply(int nx, int ny, const T* __restrict__ u, T* __restrict__ Lu,
-                                                      const T* __restrict__ c, T scale) {
+                                                      const T* __restrict__ c, int pitch, T scale) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
     const int64_t N = (int64_t)nx * ny, q = (int64_t)j * nx + i, v = blockIdx.z;
     T rj;
-    const T jl = mapped_jlap<T>(u + v * N, c, N, nx, ny, i, j, q, rj);
+    const T jl = mapped_jlap<T>(u + v * N, c, pitch, (int64_t)pitch * ny, nx, ny, i, j, q, rj);
     Lu[v * N + q] = scale * rj * jl;
 }
 
-// first step: D^1 = (dt^2/2) L V, W^1 = V + D^1, out = c0 V + c1 W^1
+// first step: D^1 = (dt^2/2) L V, W^1 = V + D^1, out = c0 V + c1 W^1; D^1 and
+// W^1 have row pitch fpitch
 template <typename T>
 __global__ void __launch_bounds__(128) k_mapped_first(int nx, int ny, const T* __restrict__ vin, T* __restrict__ D1,
                                                       T* __restrict__ W1, T* __restrict__ vout,
-                                                      const T* __restrict__ c, T half_dt2, T c0, T c1,
-                                                      int64_t fstride) {
+                                                      const T* __restrict__ c, int pitch, T half_dt2, T c0, T c1,
+                                                      int64_t fstride, int fpitch) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
     const int64_t N = (int64_t)nx * ny, q = (int64_t)j * nx + i, v = blockIdx.z;
     const T x = vin[v * N + q];
     T rj;
-    const T jl = mapped_jlap<T>(vin + v * N, c, N, nx, ny, i, j, q, rj);
+    const T jl = mapped_jlap<T>(vin + v * N, c, pitch, (int64_t)pitch * ny, nx, ny, i, j, q, rj);
     const T d = half_dt2 * rj * jl;
     const T w1 = x + d;
-    D1[v * fstride + q] = d;
-    W1[v * fstride + q] = w1;
+    const int64_t f = v * fstride + (int64_t)j * fpitch + i;
+    D1[f] = d;
+    W1[f] = w1;
     vout[v * N + q] = c0 * x + c1 * w1;
 }
 
@@ -277,13 +260,14 @@ __global__ void __launch_bounds__(128) k_mapped_first(int nx, int ny, const T* _
 template <typename T>
 __global__ void __launch_bounds__(128) k_mapped_step(int nx, int ny, const T* __restrict__ W, T* __restrict__ D,
                                                      T* __restrict__ Wout, T* __restrict__ acc,
-                                                     const T* __restrict__ c, T dt2, T cn, int64_t fstride) {
+                                                     const T* __restrict__ c, int pitch, T dt2, T cn,
+                                                     int64_t fstride) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
     const int64_t N = (int64_t)nx * ny, q = (int64_t)j * nx + i, v = blockIdx.z;
     const int64_t f = v * fstride + q;
     T rj;
-    const T jl = mapped_jlap<T>(W + v * fstride, c, N, nx, ny, i, j, q, rj);
+    const T jl = mapped_jlap<T>(W + v * fstride, c, pitch, (int64_t)pitch * ny, nx, ny, i, j, q, rj);
     const T d = D[f] + dt2 * rj * jl;
     const T wn = W[f] + d;
     D[f] = d;
@@ -305,7 +289,7 @@ ew_status mapped_apply_L(const GridGeom& g, const T* u, T* Lu, int nvec, double 
     EW_TRY(mapped_check(g, nvec));
     const T* c = nullptr;
     EW_TRY(mapped_device<T>(g, &c, nullptr));
-    k_mapped_apply<T><<<mgrid(g, nvec), 128, 0, st>>>((int)g.n[0], (int)g.n[1], u, Lu, c, T(scale));
+    k_mapped_apply<T><<<mgrid(g, nvec), 128, 0, st>>>((int)g.n[0], (int)g.n[1], u, Lu, c, (int)pitch2d(g.n[0]), T(scale));
     EW_CUDA_TRY(cudaGetLastError());
     count_launch();
     return EW_OK;
@@ -314,35 +298,41 @@ template ew_status mapped_apply_L<float>(const GridGeom&, const float*, float*, 
 template ew_status mapped_apply_L<double>(const GridGeom&, const double*, double*, int, double, cudaStream_t);
 
 template <typename T>
-ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* vin, T* vout, int nvec, T* fields,
-                            cudaStream_t st) {
+ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* cdev, const T* vin, T* vout, int nvec,
+                            T* fields, cudaStream_t st) {
     EW_TRY(mapped_check(g, nvec));
     const T* c = nullptr;
     EW_TRY(mapped_device<T>(g, &c, nullptr));
-    const int64_t fstride = field_stride(g.N);
-    T* F[3];
-    for (int q = 0; q < 3; ++q) F[q] = fields + (int64_t)q * nvec * fstride;
-    const int nx = (int)g.n[0], ny = (int)g.n[1];
+    const int64_t fstride = wave_field_stride(g);
+    T* F[4];
+    for (int q = 0; q < 4; ++q) F[q] = fields + (int64_t)q * nvec * fstride;
+    const int nx = (int)g.n[0], ny = (int)g.n[1], pitch = (int)pitch2d(g.n[0]);
     const dim3 grid = mgrid(g, nvec);
-    k_mapped_first<T><<<grid, 128, 0, st>>>(nx, ny, vin, F[0], F[1], vout, c, T(0.5 * plan.dt * plan.dt),
-                                            T(plan.cn(0)), T(plan.cn(1)), fstride);
+    constexpr bool blocked = sizeof(T) == 4;
+    k_mapped_first<T><<<grid, 128, 0, st>>>(nx, ny, vin, F[0], F[1], vout, c, pitch, T(0.5 * plan.dt * plan.dt),
+                                            T(plan.cn(0)), T(plan.cn(1)), fstride, blocked ? pitch : nx);
     EW_CUDA_TRY(cudaGetLastError());
     count_launch();
     const T dt2 = T(plan.dt * plan.dt);
-    int cur = 1, nxt = 2;
-    for (int64_t L = 1; L < plan.Nt; ++L) {
-        cudaEvent_t ev = fused_begin(st);
-        k_mapped_step<T><<<grid, 128, 0, st>>>(nx, ny, F[cur], F[0], F[nxt], vout, c, dt2, T(plan.cn(L + 1)), fstride);
-        EW_CUDA_TRY(cudaGetLastError());
-        fused_end(ev, st, g.N * nvec, g.N * nvec);
-        std::swap(cur, nxt);
+    if constexpr (blocked) {
+        return mapped_advance(g, plan, c, cdev, F, vout, nvec, fstride, dt2, st);
+    } else {
+        int cur = 1, nxt = 2;
+        for (int64_t L = 1; L < plan.Nt; ++L) {
+            cudaEvent_t ev = fused_begin(st);
+            k_mapped_step<T><<<grid, 128, 0, st>>>(nx, ny, F[cur], F[0], F[nxt], vout, c, pitch, dt2,
+                                                   T(plan.cn(L + 1)), fstride);
+            EW_CUDA_TRY(cudaGetLastError());
+            fused_end(ev, st, g.N * nvec, g.N * nvec);
+            std::swap(cur, nxt);
+        }
+        return EW_OK;
     }
-    return EW_OK;
 }
-template ew_status mapped_wave_solve<float>(const GridGeom&, const FilterPlan&, const float*, float*, int, float*,
-                                            cudaStream_t);
-template ew_status mapped_wave_solve<double>(const GridGeom&, const FilterPlan&, const double*, double*, int,
-                                             double*, cudaStream_t);
+template ew_status mapped_wave_solve<float>(const GridGeom&, const FilterPlan&, const float*, const float*, float*, int,
+                                            float*, cudaStream_t);
+template ew_status mapped_wave_solve<double>(const GridGeom&, const FilterPlan&, const double*, const double*, double*,
+                                             int, double*, cudaStream_t);
 
 // out = sqrt(J)^e in, in == out allowed
 template <typename T>

@@ -319,7 +319,7 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
         // double-FP32 pairs: 2D boxes only (the blocked 2D, one-CTA and one-step kernels)
         if (g.map || g.dim != 2) return set_error(EW_EUNSUPPORTED, "double-FP32 fields: 2D boxes only");
     } else {
-        if (g.map) return mapped_wave_solve<T>(g, plan, vin, vout, nvec, fields, st);  // one step per launch
+        if (g.map) return mapped_wave_solve<T>(g, plan, cdev, vin, vout, nvec, fields, st);
     }
     // the variant override EW_TB2D_VARIANT (a tuning and testing hook) selects a
     // blocked kernel, so it also bypasses the on-chip path of small grids
