@@ -208,6 +208,13 @@ template <typename T>
 ew_status tb3d_advance(const GridGeom& g, const FilterPlan& plan, const T* cdev, T* const* F, int* prv, int* cur,
                        int64_t L, T* acc, int nvec, int64_t fstride, int tb, cudaStream_t st);
 
+// the FP32 form for both orders (ew_tb3d_wide.cu)
+bool tb3d_wide_fits(const GridGeom& g, int nvec);
+ew_status tb3d_wide_tune(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
+                         int nvec, int64_t fstride, cudaStream_t st);
+ew_status tb3d_wide_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, int* prv,
+                            int* cur, int64_t L, float* acc, int nvec, int64_t fstride, int tb, cudaStream_t st);
+
 // register-blocked persistent form of the 2D FP32 blocked step (ew_rb2d.cu)
 struct Rb2dDesc {
     void* fn;      // boxes with Dirichlet faces only

@@ -332,7 +332,15 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
     const bool blocked = g.dim == 2 && temporal_block != 1;
     // the tuner writes the spare fields and the filter sum, so it runs before the first step
     if (blocked && temporal_block == 0) EW_TRY(tb2d_tune<T>(g, plan, cdev, F, vout, nvec, fstride, st));
-    if constexpr (!std::is_same<T, dd>::value)
+    if constexpr (std::is_same<T, float>::value) {
+        if (temporal_block != 1 && tb3d_wide_fits(g, nvec)) {
+            int prv = 0, cur = 1;
+            if (temporal_block == 0) EW_TRY(tb3d_wide_tune(g, plan, cdev, F, vout, nvec, fstride, st));
+            EW_TRY(first_step<T>(g, vin, F[0], F[1], vout, plan, nvec, fstride, st, g.n[0]));
+            return tb3d_wide_advance(g, plan, cdev, F, &prv, &cur, 1, vout, nvec, fstride, temporal_block, st);
+        }
+    }
+    if constexpr (std::is_same<T, double>::value)
         if (g.dim == 3 && g.order == 2 && temporal_block == 0)
             EW_TRY(tb3d_tune<T>(g, plan, cdev, F, vout, nvec, fstride, st));
     // F[0] = D^n, F[1] = W^n; the unblocked steps write W^{n+1} to F[2] and swap
@@ -343,7 +351,7 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
         int prv = 0, cur = 1;
         return tb2d_advance<T>(g, plan, cdev, F, &prv, &cur, 1, vout, nvec, fstride, temporal_block, st);
     }
-    if constexpr (!std::is_same<T, dd>::value)
+    if constexpr (std::is_same<T, double>::value)
         if (g.dim == 3 && g.order == 2 && temporal_block != 1) {
             int prv = 0, cur = 1;
             return tb3d_advance<T>(g, plan, cdev, F, &prv, &cur, 1, vout, nvec, fstride, temporal_block, st);

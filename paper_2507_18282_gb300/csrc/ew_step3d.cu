@@ -1,5 +1,6 @@
 // ew_step3d.cu -- one fused leapfrog + filter step on 3D grids, streamed
-// along z (eqs. explicitScheme, filterQuadrature).
+// along z (eqs. explicitScheme, filterQuadrature): FP64 grids of fourth order,
+// and every grid at one step a launch.
 //
 //   D^{n+1} = D^n + dt^2 L_h W^n (in place),  W^{n+1} = W^n + D^{n+1},  acc += c W^{n+1}
 //   (D^n = W^n - W^{n-1}: the summed form of the leapfrog recurrence)
