@@ -202,7 +202,7 @@ ew_status check_grid(const ew_grid* g) {
 
 size_t elem_size(const ew_grid* g) { return g->prec == EW_FP32 ? 4 : 8; }
 
-static ew_status pinned(ew_grid* g, size_t bytes, void** out) {
+ew_status pinned(ew_grid* g, size_t bytes, void** out) {
     if (g->host_pinned_bytes < bytes) {
         if (g->host_pinned) cudaFreeHost(g->host_pinned);
         g->host_pinned = nullptr;

@@ -192,6 +192,8 @@ ew_status plan_filter(const GridGeom& g, const ew_filter_params* p, FilterPlan* 
 // the grid is usable on the current device (binds it on first use); bytes of one vector element
 ew_status check_grid(const ew_grid* g);
 size_t elem_size(const ew_grid* g);
+// the grid's page-locked staging buffer, at least `bytes` long
+ew_status pinned(ew_grid* g, size_t bytes, void** out);
 
 // --- kernels launchers (ew_stencil.cu) ------------------------------------
 template <typename T>
@@ -345,6 +347,8 @@ constexpr int kReduceBlocks = 304;
 template <typename T>
 ew_status launch_dots(const T* x, const T* y, int64_t N, int nvec, double* part, double* out,
                       cudaStream_t st);
+// out[j] = sum of vector j's nblocks partial sums
+ew_status launch_finish_sum(const double* part, int nblocks, int nvec, double* out, cudaStream_t st);
 // out[j] = max_i |x_j[i] + s_j y_j[i]| (s on device) and max_i |y_j[i]|
 template <typename T>
 ew_status launch_resid_inf(const T* Lx, const T* x, int64_t N, int nvec, const double* lam2,

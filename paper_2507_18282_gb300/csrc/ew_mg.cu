@@ -17,7 +17,8 @@
 //               FP32, ew_smoother_comp.cu)
 //   restriction full weighting, tensor product of (1/4, 1/2, 1/4)
 //   prolongation (multi)linear interpolation, zero on the boundary
-//   coarsest    conjugate gradients in one CTA (M is SPD)
+//   coarsest    by sine transforms up to six points per axis, else conjugate
+//               gradients (M is SPD), in one CTA
 //
 // Implicit wave-solve (one application of S):
 //   M W^1 = W^0;  M y = 2 W^n, W^{n+1} = y - W^{n-1};  V_out = sum c_n W^n
@@ -25,7 +26,9 @@
 // initial guess y = 2 W^n (W^1 = W^0 for the first step) or, with
 // guess = 1, from the previous system's solution.
 // Kernels: 3D levels run their stencil operations 2.5D blocked
-// (k_mg_plane3d), 2D levels one thread per point.
+// (k_mg_plane3d), 2D levels several sweeps a launch on tiles, and the smallest
+// levels together in one launch (ew_mg_fused.cu).  1023^2 order 2 in FP64,
+// red-black, 87 cycles of a wave-solve: 58.9 -> 24.2 ms (8044 launches -> 1606).
 #include <math.h>
 #include <stdlib.h>
 
@@ -33,6 +36,7 @@
 #include <vector>
 
 #include "ew_internal.h"
+#include "ew_mg.cuh"
 #include "ew_stencil_dev.cuh"
 
 namespace ew {
@@ -83,27 +87,6 @@ static dim3 pt_grid(int64_t nx, int64_t ny, int64_t nz) {
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
-// r = b - M x = b - x + a L x   (sa carries the scale a)
-template <typename T, int DIM, int ORDER>
-__global__ void k_mg_resid(int64_t nx, int64_t ny, int64_t nz, const T* __restrict__ x, const T* __restrict__ b,
-                           T* __restrict__ r, Stencil<T> sa) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nx) return;
-    const int64_t j = blockIdx.y, k = blockIdx.z, q = (k * ny + j) * nx + i;
-    r[q] = (b[q] - x[q]) + lap_global<T, DIM, ORDER>(x, sa, q, i, j, k, nx, ny, nz);
-}
-
-// x_out = x_in + wd (b - M x_in), wd = w / D
-template <typename T, int DIM, int ORDER>
-__global__ void k_mg_jacobi(int64_t nx, int64_t ny, int64_t nz, const T* __restrict__ x, const T* __restrict__ b,
-                            T* __restrict__ xo, Stencil<T> sa, T wd) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nx) return;
-    const int64_t j = blockIdx.y, k = blockIdx.z, q = (k * ny + j) * nx + i;
-    T r = (b[q] - x[q]) + lap_global<T, DIM, ORDER>(x, sa, q, i, j, k, nx, ny, nz);
-    xo[q] = x[q] + wd * r;
-}
-
 // multi-colour Gauss-Seidel, in place: the points of one colour take
 // x += (b - M x) * inv_d, M_ii = 1 / inv_d.  Second order: red-black, colour
 // (i + j + k) & 1.  Fourth order (offsets of 1 and 2 along one axis): three
@@ -114,17 +97,6 @@ __global__ void k_mg_jacobi(int64_t nx, int64_t ny, int64_t nz, const T* __restr
 template <int ORDER>
 __device__ __forceinline__ int mg_colour(int64_t i, int64_t j, int64_t k) {
     return ORDER == 2 ? (int)((i + j + k) & 1) : (int)((i + j + k) % 3);
-}
-
-template <typename T, int ORDER>
-__global__ void k_mg_rbgs(int64_t nx, int64_t ny, T* __restrict__ x, const T* __restrict__ b, Stencil<T> sa, T inv_d,
-                          int colour) {  // 2D levels (3D: k_mg_plane3d, MODE 2)
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= nx) return;
-    const int64_t j = blockIdx.y, q = j * nx + i;
-    if (mg_colour<ORDER>(i, j, 0) != colour) return;
-    const T r = (b[q] - x[q]) + lap_global<T, 2, ORDER>(x, sa, q, i, j, 0, nx, ny, 1);
-    x[q] = x[q] + inv_d * r;
 }
 
 // ---------------------------------------------------------------------------
@@ -307,20 +279,20 @@ __device__ __forceinline__ T get0(const T* __restrict__ v, int64_t i, int64_t j,
 }
 
 // full weighting: bc(I) = sum_o w(o) r(2I + 1 + o); x_c = 0
-template <typename T, int DIM>
-__global__ void k_mg_restrict(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int64_t cy, int64_t cz,
+template <typename T>
+__global__ void k_mg_restrict3d(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int64_t cy, int64_t cz,
                               const T* __restrict__ r, T* __restrict__ bc, T* __restrict__ xc) {
     const T w[3] = {T(0.25), T(0.5), T(0.25)};
     {
         const int64_t I = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
         if (I >= cx) return;
         const int64_t J = blockIdx.y, K = blockIdx.z, q = (K * cy + J) * cx + I;
-        int64_t fi = 2 * I + 1, fj = 2 * J + 1, fk = DIM == 3 ? 2 * K + 1 : 0;
+        int64_t fi = 2 * I + 1, fj = 2 * J + 1, fk = 2 * K + 1;
         T s = T(0);
-        for (int oz = (DIM == 3 ? -1 : 0); oz <= (DIM == 3 ? 1 : 0); ++oz)
+        for (int oz = -1; oz <= 1; ++oz)
             for (int oy = -1; oy <= 1; ++oy)
                 for (int ox = -1; ox <= 1; ++ox) {
-                    T wt = w[ox + 1] * w[oy + 1] * (DIM == 3 ? w[oz + 1] : T(1));
+                    T wt = w[ox + 1] * w[oy + 1] * w[oz + 1];
                     s += wt * get0(r, fi + ox, fj + oy, fk + oz, fx, fy, fz);
                 }
         bc[q] = s;
@@ -329,8 +301,8 @@ __global__ void k_mg_restrict(int64_t fx, int64_t fy, int64_t fz, int64_t cx, in
 }
 
 // x_f += P e_c (linear interpolation per axis)
-template <typename T, int DIM>
-__global__ void k_mg_prolong(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int64_t cy, int64_t cz,
+template <typename T>
+__global__ void k_mg_prolong3d(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int64_t cy, int64_t cz,
                              const T* __restrict__ ec, T* __restrict__ xf) {
     {
         const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -342,13 +314,13 @@ __global__ void k_mg_prolong(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int
         // weights leaves the same terms in the same order
         const int64_t ci = (i & 1) ? (i - 1) / 2 : i / 2 - 1;
         const int64_t cj = (j & 1) ? (j - 1) / 2 : j / 2 - 1;
-        const int64_t ck = DIM == 2 ? 0 : ((k & 1) ? (k - 1) / 2 : k / 2 - 1);
+        const int64_t ck = (k & 1) ? (k - 1) / 2 : k / 2 - 1;
         const T wi[2] = {(i & 1) ? T(1) : T(0.5), (i & 1) ? T(0) : T(0.5)};
         const T wj[2] = {(j & 1) ? T(1) : T(0.5), (j & 1) ? T(0) : T(0.5)};
-        const T wk[2] = {(DIM == 2 || (k & 1)) ? T(1) : T(0.5), (DIM == 2 || (k & 1)) ? T(0) : T(0.5)};
+        const T wk[2] = {(k & 1) ? T(1) : T(0.5), (k & 1) ? T(0) : T(0.5)};
         T s = T(0);
 #pragma unroll
-        for (int c3 = 0; c3 < (DIM == 3 ? 2 : 1); ++c3)
+        for (int c3 = 0; c3 < 2; ++c3)
 #pragma unroll
             for (int c2 = 0; c2 < 2; ++c2)
 #pragma unroll
@@ -359,63 +331,14 @@ __global__ void k_mg_prolong(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int
     }
 }
 
-// coarsest level: CG in one CTA, all vectors in shared memory (N <= kCoarseMax)
-constexpr int kCoarseMax = 2048;
+// coarsest level in a launch of its own (ew_mg.cuh)
 constexpr int kCoarseThreads = 512;
-
-template <typename T>
-__device__ T block_dot(const T* a, const T* b, int N, T* red) {
-    T s = T(0);
-    for (int q = threadIdx.x; q < N; q += blockDim.x) s += a[q] * b[q];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    T t = T(0);
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    __syncthreads();
-    return t;
-}
 
 template <typename T, int DIM, int ORDER>
 __global__ void __launch_bounds__(kCoarseThreads)
-    k_mg_coarse_cg(int nx, int ny, int nz, const T* __restrict__ b, T* __restrict__ x, Stencil<T> sa, T rtol,
-                   int maxit) {
+    k_mg_coarse_cg(int nx, int ny, int nz, const T* b, T* x, Stencil<T> sa, T rtol, int maxit) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = nx * ny * nz;
-    T* sx = reinterpret_cast<T*>(smem_raw);
-    T* sr = sx + N;
-    T* sp = sr + N;
-    T* sq = sp + N;
-    T* red = sq + N;
-    for (int q = threadIdx.x; q < N; q += blockDim.x) {
-        sx[q] = T(0);
-        sr[q] = b[q];
-        sp[q] = b[q];
-    }
-    __syncthreads();
-    T rr = block_dot(sr, sr, N, red);
-    const T stop = rtol * rtol * rr;
-    for (int it = 0; it < maxit && rr > stop && rr > T(0); ++it) {
-        for (int q = threadIdx.x; q < N; q += blockDim.x) {
-            int i = q % nx, t = q / nx, j = t % ny, k = t / ny;
-            sq[q] = sp[q] - lap_global<T, DIM, ORDER>(sp, sa, q, i, j, k, nx, ny, nz);  // M p
-        }
-        __syncthreads();
-        T pq = block_dot(sp, sq, N, red);
-        if (!(pq > T(0))) break;
-        T alpha = rr / pq;
-        for (int q = threadIdx.x; q < N; q += blockDim.x) {
-            sx[q] += alpha * sp[q];
-            sr[q] -= alpha * sq[q];
-        }
-        __syncthreads();
-        T rr2 = block_dot(sr, sr, N, red);
-        T beta = rr2 / rr;
-        rr = rr2;
-        for (int q = threadIdx.x; q < N; q += blockDim.x) sp[q] = sr[q] + beta * sp[q];
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < N; q += blockDim.x) x[q] = sx[q];
+    coarse_cg<T, DIM, ORDER>(nx, ny, nz, b, x, sa, rtol, maxit, reinterpret_cast<T*>(smem_raw));
 }
 
 template <typename T>
@@ -539,19 +462,7 @@ struct MGSolver {
         return 1.0 + a * s;
     }
 
-// 2D levels: one thread per point (3D levels go through k_mg_plane3d)
-#define EW_MG_DISPATCH2D(KERN, GEOM, ...)                                                                \
-    do {                                                                                                 \
-        const GridGeom& g_ = (GEOM);                                                                     \
-        dim3 grid_ = pt_grid(g_.n[0], g_.n[1], 1), blk_(pt_threads(g_.n[0]));                            \
-        if (g_.order == 2)                                                                               \
-            KERN<T, 2, 2><<<grid_, blk_, 0, st>>>(g_.n[0], g_.n[1], 1, __VA_ARGS__);                     \
-        else                                                                                             \
-            KERN<T, 2, 4><<<grid_, blk_, 0, st>>>(g_.n[0], g_.n[1], 1, __VA_ARGS__);                     \
-        count_launch();                                                                                  \
-    } while (0)
-
-    // 3D levels: the 2.5D-blocked stencil kernel; 2D levels: one thread per point
+    // 3D levels: the 2.5D-blocked stencil kernel
     int nsm = 0, pl_occ[2] = {1, 1};  // SMs; resident plane-kernel CTAs a SM (order 2, order 4)
     template <int MODE>
     void plane3d(const GridGeom& g_, const T* x, const T* b, T* out, const Stencil<T>& sa, T wd, int colour) {
@@ -569,13 +480,9 @@ struct MGSolver {
                                                                               colour);
         count_launch();
     }
-    void resid(int L, const Stencil<T>& sa) {
-        if (lv[L].dim == 3)
-            plane3d<0>(lv[L], X[L], B[L], R[L], sa, T(0), 0);
-        else
-            EW_MG_DISPATCH2D(k_mg_resid, lv[L], X[L], B[L], R[L], sa);
-    }
+    void resid(int L, const Stencil<T>& sa) { plane3d<0>(lv[L], X[L], B[L], R[L], sa, T(0), 0); }
 
+    // 3D levels
     ew_status smooth(int L, int steps) {
         Stencil<T> sa = make_stencil<T>(lv[L], a);
         for (int s = 0; s < steps; ++s) {
@@ -589,39 +496,78 @@ struct MGSolver {
                 }
                 EW_TRY(smoother_apply<T>(lv[L], p->weights_dev + (size_t)L * 432, R[L], X[L], st));
             } else if (p->red_black) {
-                // M_ii = 1 - c0 of the stored (consistent) stencil of a L_h
-                const T inv_d = (T)(1.0 / (1.0 - (double)sa.c0));
-                const GridGeom& g_ = lv[L];
-                dim3 grid_ = pt_grid(g_.n[0], g_.n[1], 1), blk_(pt_threads(g_.n[0]));
-                const int ncol = g_.order == 2 ? 2 : 3;
-                for (int colour = 0; colour < ncol; ++colour) {
-                    // one launch per colour: 3D levels the 2.5D kernel, 2D levels one thread per point
-                    if (g_.dim == 3)
-                        plane3d<2>(g_, X[L], B[L], X[L], sa, inv_d, colour);
-                    else if (g_.order == 2)
-                        k_mg_rbgs<T, 2><<<grid_, blk_, 0, st>>>(g_.n[0], g_.n[1], X[L], B[L], sa, inv_d, colour);
-                    else
-                        k_mg_rbgs<T, 4><<<grid_, blk_, 0, st>>>(g_.n[0], g_.n[1], X[L], B[L], sa, inv_d, colour);
-                    if (g_.dim == 2) count_launch();
-                }
+                // 3D levels: one launch per colour
+                const int ncol = lv[L].order == 2 ? 2 : 3;
+                for (int colour = 0; colour < ncol; ++colour)
+                    plane3d<2>(lv[L], X[L], B[L], X[L], sa, weight(L, sa), colour);
             } else {
-                T wd = (T)(wJ / diag(L));
-                if (lv[L].dim == 3)
-                    plane3d<1>(lv[L], X[L], B[L], Tm[L], sa, wd, 0);
-                else
-                    EW_MG_DISPATCH2D(k_mg_jacobi, lv[L], X[L], B[L], Tm[L], sa, wd);
+                plane3d<1>(lv[L], X[L], B[L], Tm[L], sa, weight(L, sa), 0);
                 std::swap(X[L], Tm[L]);
             }
         }
         return EW_OK;
     }
 
+    // x += weight (b - M x): w / D (Jacobi), or 1 / M_ii with M_ii = 1 - c0 of the
+    // stored (consistent) stencil of a L_h (colour sweeps)
+    T weight(int L, const Stencil<T>& sa) const {
+        return p->red_black ? (T)(1.0 / (1.0 - (double)sa.c0)) : (T)(wJ / diag(L));
+    }
+
+    // 2D levels: `steps` sweeps, a few a launch; the first launch adds the
+    // prolongation of the coarse iterate when `correct`
+    ew_status smooth2d(int L, int steps, bool correct) {
+        const Stencil<T> sa = make_stencil<T>(lv[L], a);
+        const int most = mg_smooth2d_sweeps<T>(lv[L].order, p->red_black != 0);
+        while (steps > 0) {
+            const int ns = std::min(steps, most);
+            EW_TRY(mg_smooth2d<T>(lv[L], X[L], B[L], Tm[L], sa, weight(L, sa), p->red_black != 0, ns,
+                                  correct ? X[L + 1] : nullptr, correct ? &lv[L + 1] : nullptr, st));
+            std::swap(X[L], Tm[L]);
+            correct = false;
+            steps -= ns;
+        }
+        return EW_OK;
+    }
+
+    // The levels from L down to the coarsest and back in one launch of one CTA,
+    // once they are small: up to 31^2 points in FP64 (63^2 would take that SM's
+    // FP64 units 37 us, three launches 15-20 us), 4096 in FP32
+    bool bottom_fits(int L) const {
+        if (L < p->learned_levels || L == 0 || nlev - L > kMgBottomLevels) return false;
+        if (lv[L].N > (sizeof(T) == 8 ? 1024 : 4096)) return false;
+        int64_t n[kMgBottomLevels];
+        for (int l = L; l < nlev; ++l) n[l - L] = lv[l].N;
+        return mg_bottom_smem<T>(n, nlev - L) <= 200 * 1024;
+    }
+    ew_status bottom(int L) {
+        MgBottom<T> m;
+        m.nlev = nlev - L;
+        m.pre = p->pre;
+        m.post = p->post;
+        m.colours = p->red_black ? (lv[L].order == 2 ? 2 : 3) : 0;
+        m.cg_rtol = cg_rtol();
+        m.cg_maxit = cg_maxit(lv[nlev - 1]);
+        m.cg_off = 0;
+        m.b = B[L];
+        m.x = X[L];
+        for (int l = L; l < nlev; ++l) {
+            MgBottomLevel<T>& q = m.lv[l - L];
+            for (int d = 0; d < 3; ++d) q.n[d] = (int)lv[l].n[d];
+            q.sa = make_stencil<T>(lv[l], a);
+            q.wd = weight(l, q.sa);
+        }
+        return mg_bottom<T>(lv[L].dim, lv[L].order, m, st);
+    }
+
+    static T cg_rtol() { return sizeof(T) == 4 ? T(1e-7) : T(1e-14); }
+    static int cg_maxit(const GridGeom& c) { return (int)std::min<int64_t>(4 * c.N + 10, 4000); }
     ew_status coarse(int L) {
         Stencil<T> sa = make_stencil<T>(lv[L], a);
         const GridGeom& c = lv[L];
-        size_t smem = sizeof(T) * (4 * (size_t)c.N + 32);
-        T rtol = sizeof(T) == 4 ? T(1e-7) : T(1e-14);
-        int maxit = (int)std::min<int64_t>(4 * c.N + 10, 4000);
+        size_t smem = coarse_cg_smem<T>(c.N);
+        const T rtol = cg_rtol();
+        const int maxit = cg_maxit(c);
         if (c.dim == 2 && c.order == 2)
             k_mg_coarse_cg<T, 2, 2><<<1, kCoarseThreads, smem, st>>>((int)c.n[0], (int)c.n[1], 1, B[L], X[L], sa, rtol, maxit);
         else if (c.dim == 2)
@@ -636,26 +582,26 @@ struct MGSolver {
     }
 
     ew_status vcycle(int L) {
+        if (bottom_fits(L)) return bottom(L);
         if (L == nlev - 1) return coarse(L);
-        EW_TRY(smooth(L, p->pre));
-        Stencil<T> sa = make_stencil<T>(lv[L], a);
-        resid(L, sa);
         const GridGeom &f = lv[L], &c = lv[L + 1];
-        const int fz = f.dim == 3 ? (int)f.n[2] : 1, cz = f.dim == 3 ? (int)c.n[2] : 1;
-        if (f.dim == 2)
-            k_mg_restrict<T, 2><<<pt_grid(c.n[0], c.n[1], cz), pt_threads(c.n[0]), 0, st>>>(
-                f.n[0], f.n[1], fz, c.n[0], c.n[1], cz, R[L], B[L + 1], X[L + 1]);
-        else
-            k_mg_restrict<T, 3><<<pt_grid(c.n[0], c.n[1], cz), pt_threads(c.n[0]), 0, st>>>(
-                f.n[0], f.n[1], fz, c.n[0], c.n[1], cz, R[L], B[L + 1], X[L + 1]);
+        const Stencil<T> sa = make_stencil<T>(f, a);
+        if (f.dim == 2) {
+            EW_TRY(smooth2d(L, p->pre, false));
+            EW_TRY(mg_resid_restrict2d<T>(f, c, X[L], B[L], B[L + 1], X[L + 1], sa, st));
+            EW_TRY(vcycle(L + 1));
+            if (p->post > 0) return smooth2d(L, p->post, true);
+            // no smoothing afterwards: the correction alone
+            return mg_prolong2d<T>(f, c, X[L + 1], X[L], st);
+        }
+        EW_TRY(smooth(L, p->pre));
+        resid(L, sa);
+        k_mg_restrict3d<T><<<pt_grid(c.n[0], c.n[1], c.n[2]), pt_threads(c.n[0]), 0, st>>>(
+            f.n[0], f.n[1], f.n[2], c.n[0], c.n[1], c.n[2], R[L], B[L + 1], X[L + 1]);
         count_launch();
         EW_TRY(vcycle(L + 1));
-        if (f.dim == 2)
-            k_mg_prolong<T, 2><<<pt_grid(f.n[0], f.n[1], fz), pt_threads(f.n[0]), 0, st>>>(
-                f.n[0], f.n[1], fz, c.n[0], c.n[1], cz, X[L + 1], X[L]);
-        else
-            k_mg_prolong<T, 3><<<pt_grid(f.n[0], f.n[1], fz), pt_threads(f.n[0]), 0, st>>>(
-                f.n[0], f.n[1], fz, c.n[0], c.n[1], cz, X[L + 1], X[L]);
+        k_mg_prolong3d<T><<<pt_grid(f.n[0], f.n[1], f.n[2]), pt_threads(f.n[0]), 0, st>>>(
+            f.n[0], f.n[1], f.n[2], c.n[0], c.n[1], c.n[2], X[L + 1], X[L]);
         count_launch();
         EW_TRY(smooth(L, p->post));
         EW_CUDA_TRY(cudaGetLastError());
@@ -669,16 +615,26 @@ struct MGSolver {
         return EW_OK;
     }
 
-    // ||v||_2 of a finest-level vector (FP64 reduction, synchronises)
-    ew_status norm2(const T* v, double* out) {
-        EW_TRY(gr->reduce.reserve(sizeof(double) * (kReduceBlocks + 8)));
+    // ||B[0]||_2 or ||B[0] - M X[0]||_2 (FP64 reduction, synchronises)
+    ew_status norm2(bool residual, double* out) {
+        constexpr int nb = 2 * kReduceBlocks;
+        EW_TRY(gr->reduce.reserve(sizeof(double) * (nb + 8)));
         double* dpart = (double*)gr->reduce.ptr;
-        double* dres = dpart + kReduceBlocks;
-        EW_TRY(launch_dots<T>(v, v, lv[0].N, 1, dpart, dres, st));
-        double h = 0.0;
-        EW_CUDA_TRY(cudaMemcpyAsync(&h, dres, sizeof(double), cudaMemcpyDeviceToHost, st));
+        double* dres = dpart + nb;
+        if (!residual) {
+            EW_TRY(launch_dots<T>(B[0], B[0], lv[0].N, 1, dpart, dres, st));
+        } else if (lv[0].dim == 2) {
+            EW_TRY(mg_resid_norm2d<T>(lv[0], X[0], B[0], make_stencil<T>(lv[0], a), dpart, nb, st));
+            EW_TRY(launch_finish_sum(dpart, nb, 1, dres, st));
+        } else {
+            resid(0, make_stencil<T>(lv[0], a));
+            EW_TRY(launch_dots<T>(R[0], R[0], lv[0].N, 1, dpart, dres, st));
+        }
+        void* hp = nullptr;  // page-locked: a copy into pageable memory is staged by the driver
+        EW_TRY(pinned(gr, sizeof(double), &hp));
+        EW_CUDA_TRY(cudaMemcpyAsync(hp, dres, sizeof(double), cudaMemcpyDeviceToHost, st));
         EW_CUDA_TRY(cudaStreamSynchronize(st));
-        *out = sqrt(h);
+        *out = sqrt(*(const double*)hp);
         return EW_OK;
     }
 
@@ -690,15 +646,13 @@ struct MGSolver {
             return cycles(max_cycles);
         }
         double bn = 0.0;
-        EW_TRY(norm2(B[0], &bn));
-        Stencil<T> sa = make_stencil<T>(lv[0], a);
+        EW_TRY(norm2(false, &bn));
         int c = 0;
         while (c < max_cycles) {
             EW_TRY(vcycle(0));
             ++c;
-            resid(0, sa);
             double rk = 0.0;
-            EW_TRY(norm2(R[0], &rk));
+            EW_TRY(norm2(true, &rk));
             if (rk <= rtol * bn) break;
         }
         *used = c;
@@ -786,46 +740,17 @@ static ew_status step_mg_t(ew_grid* g, double a, const T* rhs, T* x, const ew_mg
     const int64_t N = g->geom.N;
     MGSolver<T> mg;
     EW_TRY(mg.setup(g, a, mp, st));
-    EW_TRY(g->reduce.reserve(sizeof(double) * (kReduceBlocks + 8)));
-    double* dpart = (double*)g->reduce.ptr;
-    double* dres = dpart + kReduceBlocks;
     EW_CUDA_TRY(cudaMemcpyAsync(mg.B[0], rhs, N * sizeof(T), cudaMemcpyDeviceToDevice, st));
     EW_CUDA_TRY(cudaMemcpyAsync(mg.X[0], x, N * sizeof(T), cudaMemcpyDeviceToDevice, st));
-    Stencil<T> sa = make_stencil<T>(g->geom, a);
-    auto resid_norm = [&](double* out) -> ew_status {
-        T* r = mg.R[0];
-        {
-            const GridGeom& gg = g->geom;
-            dim3 grid_ = pt_grid(gg.n[0], gg.n[1], gg.dim == 3 ? gg.n[2] : 1), blk_(pt_threads(gg.n[0]));
-            if (gg.dim == 3) {
-                mg.template plane3d<0>(gg, mg.X[0], mg.B[0], r, sa, T(0), 0);
-            } else {
-                if (gg.order == 2)
-                    k_mg_resid<T, 2, 2><<<grid_, blk_, 0, st>>>(gg.n[0], gg.n[1], 1, mg.X[0], mg.B[0], r, sa);
-                else
-                    k_mg_resid<T, 2, 4><<<grid_, blk_, 0, st>>>(gg.n[0], gg.n[1], 1, mg.X[0], mg.B[0], r, sa);
-                count_launch();
-            }
-        }
-        EW_TRY(launch_dots<T>(r, r, N, 1, dpart, dres, st));
-        double h = 0.0;
-        EW_CUDA_TRY(cudaMemcpyAsync(&h, dres, sizeof(double), cudaMemcpyDeviceToHost, st));
-        EW_CUDA_TRY(cudaStreamSynchronize(st));
-        *out = sqrt(h);
-        return EW_OK;
-    };
     double bnorm = 0.0, r0 = 0.0, rk = 0.0;
-    EW_TRY(launch_dots<T>(rhs, rhs, N, 1, dpart, dres, st));
-    EW_CUDA_TRY(cudaMemcpyAsync(&bnorm, dres, sizeof(double), cudaMemcpyDeviceToHost, st));
-    EW_CUDA_TRY(cudaStreamSynchronize(st));
-    bnorm = sqrt(bnorm);
-    EW_TRY(resid_norm(&r0));
+    EW_TRY(mg.norm2(false, &bnorm));
+    EW_TRY(mg.norm2(true, &r0));
     rk = r0;
     int c = 0;
     for (c = 0; c < mp->max_cycles; ++c) {
         if (mp->rtol > 0 && rk <= mp->rtol * bnorm) break;
         EW_TRY(mg.vcycle(0));
-        if (mp->rtol > 0 || c + 1 == mp->max_cycles) EW_TRY(resid_norm(&rk));
+        if (mp->rtol > 0 || c + 1 == mp->max_cycles) EW_TRY(mg.norm2(true, &rk));
     }
     EW_CUDA_TRY(cudaMemcpyAsync(x, mg.X[0], N * sizeof(T), cudaMemcpyDeviceToDevice, st));
     EW_CUDA_TRY(cudaStreamSynchronize(st));

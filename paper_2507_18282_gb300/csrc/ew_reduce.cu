@@ -84,6 +84,13 @@ __global__ void k_finish_max(const double* __restrict__ part, int nb, double* __
     if (threadIdx.x == 0) out[j] = s;
 }
 
+ew_status launch_finish_sum(const double* part, int nblocks, int nvec, double* out, cudaStream_t st) {
+    k_finish_sum<<<nvec, 256, 0, st>>>(part, nblocks, out);
+    EW_CUDA_TRY(cudaGetLastError());
+    count_launch();
+    return EW_OK;
+}
+
 template <typename T>
 ew_status launch_dots(const T* x, const T* y, int64_t N, int nvec, double* part, double* out,
                       cudaStream_t st) {
