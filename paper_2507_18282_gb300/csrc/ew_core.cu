@@ -239,7 +239,9 @@ static ew_status filter_apply_t(ew_grid* g, const ew_filter_params* p, const Fil
     if (p->scheme == EW_IMPLICIT) return implicit_wave_solve_any(g, plan, p, vin, vout, nvec, st);
     const T* cdev = nullptr;
     EW_TRY(upload_weights<T>(g, plan, st, &cdev));
-    EW_TRY(g->fields.reserve((size_t)4 * nvec * wave_field_stride(g->geom) * sizeof(T)));
+    size_t room = (size_t)4 * nvec * wave_field_stride(g->geom) * sizeof(T);
+    if (sizeof(T) == 4 && p->temporal_block == 0 && persist2d_fits(g->geom, nvec)) room += persist2d_room(g->geom, nvec);
+    EW_TRY(g->fields.reserve(room));
     return explicit_wave_solve<T>(g->geom, plan, cdev, vin, vout, nvec, (T*)g->fields.ptr, p->temporal_block, st);
 }
 
@@ -496,6 +498,7 @@ static ew_status rayleigh_t(ew_grid* g, const T* phi, int nvec, double* lam_host
     EW_CUDA_TRY(cudaStreamSynchronize(st));
     EW_TRY(rb2d_check_timeout());  // a register-blocked wave-solve before this point gave up a wait
     EW_TRY(tma2d_check_timeout());  // the same for a TMA-staged one
+    EW_TRY(persist2d_check_timeout());
     if (g->geom.map) EW_TRY(mapped_check_timeout());
     std::vector<double> lam2(nvec);
     for (int j = 0; j < nvec; ++j) {

@@ -201,7 +201,8 @@ ew_status launch_apply_L(const GridGeom& g, const T* u, T* Lu, int nvec, double 
                          cudaStream_t st);
 
 // one explicit wave-solve for nvec vectors; fields = 4 * N * nvec elements
-// of scratch; cdev = N_t + 1 weights (device, type T).
+// of scratch (and persist2d_room() bytes after them when temporal_block is 0
+// and persist2d_fits()); cdev = N_t + 1 weights (device, type T).
 // temporally blocked 3D second-order steps (ew_tb3d.cu)
 template <typename T>
 ew_status tb3d_tune(const GridGeom& g, const FilterPlan& plan, const T* cdev, T* const* F, T* acc, int nvec,
@@ -271,6 +272,14 @@ bool resident_fits(const GridGeom& g, int nvec);
 template <typename T>
 ew_status resident_wave_solve(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
                               cudaStream_t st);
+
+// --- 2D wave-solves that fit on the chip, one cooperative launch (ew_persist2d.cu)
+bool persist2d_fits(const GridGeom& g, int nvec);
+size_t persist2d_room(const GridGeom& g, int nvec);  // bytes it needs after the time-level fields
+ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
+                            int nvec, int64_t fstride, void* records, cudaStream_t st);
+// reads (and clears) the flag a halo exchange sets when it gives up
+ew_status persist2d_check_timeout();
 
 // --- curvilinear grids (ew_mapped.cu) ----------------------------------------
 ew_status mapped_build(int64_t n1, int64_t n2, const double* xy, MappedData* m);

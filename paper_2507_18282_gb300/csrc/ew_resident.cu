@@ -345,7 +345,7 @@ static int cluster_ctas(const GridGeom& g, int nvec) {
 // (4830 against 4938 us), and 16 x 127^2 (3554 against 8124 us).
 template <typename T>
 static bool fits_cluster(const GridGeom& g, int nvec) {
-    if (g.N > 65536 || !cluster_ctas<T>(g, nvec)) return false;
+    if (g.N > (sizeof(T) == 4 ? 32768 : 65536) || !cluster_ctas<T>(g, nvec)) return false;
     if (std::is_same<T, dd>::value) return nvec <= 16;
     if (g.N * nvec > 262144 + 2048) return false;
     return sizeof(T) == 4 || g.N <= 16384 || nvec <= 4;

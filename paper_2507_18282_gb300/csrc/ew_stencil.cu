@@ -329,6 +329,12 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
     const int64_t fstride = wave_field_stride(g);
     T* F[4];
     for (int q = 0; q < 4; ++q) F[q] = fields + (int64_t)q * nvec * fstride;
+    if constexpr (std::is_same<T, float>::value)
+        if (temporal_block == 0 && persist2d_fits(g, nvec) && !getenv("EW_TB2D_VARIANT")) {
+            EW_TRY(first_step<T>(g, vin, F[0], F[1], vout, plan, nvec, fstride, st, g.n[0]));
+            return persist2d_advance(g, plan, cdev, F, vout, nvec, fstride,
+                                     fields + 4 * (int64_t)nvec * fstride, st);
+        }
     const bool blocked = g.dim == 2 && temporal_block != 1;
     // the tuner writes the spare fields and the filter sum, so it runs before the first step
     if (blocked && temporal_block == 0) EW_TRY(tb2d_tune<T>(g, plan, cdev, F, vout, nvec, fstride, st));
