@@ -403,6 +403,9 @@ struct MGSolver {
             int dev = 0;
             EW_CUDA_TRY(cudaGetDevice(&dev));
             EW_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        }
+        f2 = sizeof(T) == 4 && mg_plane3d_f2_fits(g->geom);
+        if (g->geom.dim == 3 && !f2) {
             const int s2 = (int)PlaneRing<T, 2>::SMEM, s4 = (int)PlaneRing<T, 4>::SMEM;
             const auto A = cudaFuncAttributeMaxDynamicSharedMemorySize;
             EW_CUDA_TRY(cudaFuncSetAttribute(k_mg_plane3d<T, 2, 0>, A, s2));
@@ -464,8 +467,14 @@ struct MGSolver {
 
     // 3D levels: the 2.5D-blocked stencil kernel
     int nsm = 0, pl_occ[2] = {1, 1};  // SMs; resident plane-kernel CTAs a SM (order 2, order 4)
+    bool f2 = false;                  // FP32: the paired form (ew_mg_plane.cu)
     template <int MODE>
     void plane3d(const GridGeom& g_, const T* x, const T* b, T* out, const Stencil<T>& sa, T wd, int colour) {
+        if constexpr (sizeof(T) == 4)
+            if (f2) {
+                mg_plane3d_f2(MODE, g_, x, b, out, sa, wd, colour, nsm, st);
+                return;
+            }
         const int nx = (int)g_.n[0], ny = (int)g_.n[1], nz = (int)g_.n[2];
         const int bx = (nx + kPlBX - 1) / kPlBX, by = (ny + kPlBY - 1) / kPlBY;
         // z chunks: enough CTAs to fill the resident slots once, at least 8 planes each

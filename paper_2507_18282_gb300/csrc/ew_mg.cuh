@@ -54,6 +54,10 @@ template <typename T>
 ew_status mg_resid_restrict2d(const GridGeom& f, const GridGeom& c, const T* x, const T* b, T* bc, T* xc,
                               const Stencil<T>& sa, cudaStream_t st);
 
+// 3D FP32 levels (ew_mg_plane.cu).  mode 0: out = b - M x; 1: out = x + wd (b - M x); 2: one colour of the same in place
+bool mg_plane3d_f2_fits(const GridGeom& g);
+ew_status mg_plane3d_f2(int mode, const GridGeom& g, const float* x, const float* b, float* out,
+                        const Stencil<float>& sa, float wd, int colour, int nsm, cudaStream_t st);
 // part[0 .. nblocks): shares of |b - M x|^2
 template <typename T>
 ew_status mg_resid_norm2d(const GridGeom& g, const T* x, const T* b, const Stencil<T>& sa, double* part, int nblocks,
