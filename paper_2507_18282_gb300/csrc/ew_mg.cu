@@ -300,34 +300,53 @@ __global__ void k_mg_restrict3d(int64_t fx, int64_t fy, int64_t fz, int64_t cx, 
     }
 }
 
-// x_f += P e_c (linear interpolation per axis)
+// x_f += P e_c (linear interpolation per axis).  A thread takes the 2 x 2 x 2
+// fine points that share coarse corner (I, J, K): fine point 2 I + p along an
+// axis lies, for p = 1, on coarse point I, and for p = 0 between I - 1 and I, so
+// all eight come from the 2 x 2 x 2 coarse values around it.  Each point's terms
+// and their order are those of the tensor product over its neighbours.
+// One thread a fine point (up to eight loads and a weight product each) took
+// 109 us on 255^3, this form 62 us; 21 us is the traffic's floor.
 template <typename T>
-__global__ void k_mg_prolong3d(int64_t fx, int64_t fy, int64_t fz, int64_t cx, int64_t cy, int64_t cz,
-                             const T* __restrict__ ec, T* __restrict__ xf) {
-    {
-        const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-        if (i >= fx) return;
-        const int64_t j = blockIdx.y, k = blockIdx.z, q = (k * fy + j) * fx + i;
-        // per axis the coarse neighbours c, c + 1 and their weights: an odd fine index lies on
-        // coarse point (i - 1) / 2 (weight 1, the second weight 0), an even one between two
-        // (1/2 each); fixed trip counts keep everything in registers, and skipping the zero
-        // weights leaves the same terms in the same order
-        const int64_t ci = (i & 1) ? (i - 1) / 2 : i / 2 - 1;
-        const int64_t cj = (j & 1) ? (j - 1) / 2 : j / 2 - 1;
-        const int64_t ck = (k & 1) ? (k - 1) / 2 : k / 2 - 1;
-        const T wi[2] = {(i & 1) ? T(1) : T(0.5), (i & 1) ? T(0) : T(0.5)};
-        const T wj[2] = {(j & 1) ? T(1) : T(0.5), (j & 1) ? T(0) : T(0.5)};
-        const T wk[2] = {(k & 1) ? T(1) : T(0.5), (k & 1) ? T(0) : T(0.5)};
-        T s = T(0);
+__global__ void k_mg_prolong3d(int fx, int fy, int fz, int cx, int cy, int cz, const T* __restrict__ ec,
+                               T* __restrict__ xf) {
+    const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y, K = blockIdx.z;
+    if (2 * I >= fx) return;
+    T e[2][2][2];  // [k][j][i]: coarse points K - 1 + k, J - 1 + j, I - 1 + i, zero outside
 #pragma unroll
-        for (int c3 = 0; c3 < 2; ++c3)
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
-            for (int c2 = 0; c2 < 2; ++c2)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-                for (int c1 = 0; c1 < 2; ++c1)
-                    if (wi[c1] != T(0) && wj[c2] != T(0) && wk[c3] != T(0))
-                        s += wi[c1] * wj[c2] * wk[c3] * get0(ec, ci + c1, cj + c2, ck + c3, cx, cy, cz);
-        xf[q] += s;
+            for (int i = 0; i < 2; ++i) {
+                const int a = I - 1 + i, b = J - 1 + j, c = K - 1 + k;
+                e[k][j][i] = a >= 0 && b >= 0 && c >= 0 && a < cx && b < cy && c < cz
+                                 ? ec[((int64_t)c * cy + b) * cx + a]
+                                 : T(0);
+            }
+#pragma unroll
+    for (int pk = 0; pk < 2; ++pk) {
+        const int k = 2 * K + pk;
+        if (k >= fz) break;
+#pragma unroll
+        for (int pj = 0; pj < 2; ++pj) {
+            const int j = 2 * J + pj;
+            if (j >= fy) break;
+            T* row = xf + ((int64_t)k * fy + j) * fx + 2 * I;
+#pragma unroll
+            for (int pi = 0; pi < 2; ++pi) {
+                if (2 * I + pi >= fx) break;
+                const T w = T(1) / T((pi ? 1 : 2) * (pj ? 1 : 2) * (pk ? 1 : 2));
+                T s = T(0);
+#pragma unroll
+                for (int c = pk; c < 2; ++c)
+#pragma unroll
+                    for (int b = pj; b < 2; ++b)
+#pragma unroll
+                        for (int a = pi; a < 2; ++a) s += w * e[c][b][a];
+                row[pi] += s;
+            }
+        }
     }
 }
 
@@ -609,8 +628,12 @@ struct MGSolver {
             f.n[0], f.n[1], f.n[2], c.n[0], c.n[1], c.n[2], R[L], B[L + 1], X[L + 1]);
         count_launch();
         EW_TRY(vcycle(L + 1));
-        k_mg_prolong3d<T><<<pt_grid(f.n[0], f.n[1], f.n[2]), pt_threads(f.n[0]), 0, st>>>(
-            f.n[0], f.n[1], f.n[2], c.n[0], c.n[1], c.n[2], X[L + 1], X[L]);
+        {
+            const int64_t hx = (f.n[0] + 1) / 2;
+            const dim3 pg((unsigned)((hx + 127) / 128), (unsigned)((f.n[1] + 1) / 2), (unsigned)((f.n[2] + 1) / 2));
+            k_mg_prolong3d<T><<<pg, 128, 0, st>>>((int)f.n[0], (int)f.n[1], (int)f.n[2], (int)c.n[0], (int)c.n[1],
+                                                  (int)c.n[2], X[L + 1], X[L]);
+        }
         count_launch();
         EW_TRY(smooth(L, p->post));
         EW_CUDA_TRY(cudaGetLastError());
