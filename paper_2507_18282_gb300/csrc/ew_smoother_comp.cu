@@ -25,16 +25,25 @@
 // zero-padded outside the box; a second launch then adds, at each output on
 // a wall plane, the difference between its class's stencil and the interior
 // one (one thread per wall output, about 2.3 % of the points on 255^3).  In
-// the first, a CTA owns 128 x 8 output columns and kZ planes of them; a thread
-// owns four consecutive x outputs of one row and streams along z, keeping the
+// the first, a CTA owns 128 x 16 output columns and kZ planes of them; a thread
+// owns four consecutive x outputs of two rows and streams along z, keeping the
 // partial sums of the five output planes an input plane feeds in registers.
-// Input planes (with a halo of 2) are staged in a double-buffered shared tile,
-// one barrier per plane; the global loads of plane z + 2 are issued into
-// registers before plane z + 1 is computed, so their latency is hidden.
+// The two rows are the halves of paired multiply-adds, so that one operand
+// serves both: input rows are staged in pairs (a halo of 2 around the tile,
+// asynchronous copies into a ring of three planes, one barrier a plane), the
+// pairs one row further on are put together in registers.
+//
+// Bound: the multiply-adds (125 a point, 57 us on 255^3 at full rate) with the
+// moves of the stencil's values beside them: a paired operand has to stand in
+// two vector registers.  Measured, 255^3: scalar, 1 row of 4 a thread 110 us;
+// scalar, 2 rows 99 us (its values serve twice as many points); paired 96 us;
+// paired with the values read from shared memory 127 us (three register
+// operands a multiply-add hold the pipe up).
 #include <math.h>
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "ew_internal.h"
@@ -42,14 +51,14 @@
 namespace ew {
 
 constexpr int kCompTX = 128;  // outputs per CTA row (32 threads x 4)
-constexpr int kCompTY = 8;    // rows per CTA
+constexpr int kCompTY = 16;   // rows per CTA (8 warps x 2)
 constexpr int kCompZMin = 16;  // fewest planes per CTA (the grid's z chunks are chosen at launch)
 constexpr int kCompSX = kCompTX + 4;  // staged width (halo 2), a multiple of 4
 constexpr int kCompSY = kCompTY + 4;
 constexpr int kCompPlane = kCompSX * kCompSY;
 
-struct K125 {
-    float k[125];  // index (dz + 2) 25 + (dy + 2) 5 + (dx + 2)
+struct K125x2 {
+    float2 k[125];  // index (dz + 2) 25 + (dy + 2) 5 + (dx + 2); each value twice, the operand of a paired multiply-add
 };
 
 // class of an output coordinate on an axis: 0 low wall, 1 interior, 2 high wall, 3 both (n = 1)
@@ -57,102 +66,135 @@ __host__ __device__ __forceinline__ int comp_class(int i, int n) {
     return n == 1 ? 3 : (i == 0 ? 0 : (i == n - 1 ? 2 : 1));
 }
 
+// copy of one element into shared memory, or a zero there
+__device__ __forceinline__ void cp_async4_zfill(unsigned dst, const float* src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+
 // x += K_int * r at every output (FP32 fields, r zero outside the box); a
-// CTA owns planes [z0, z0 + zc) of its 128 x 8 columns
-__global__ void __launch_bounds__(256, 4)
-    k_smoother_comp(int nx, int ny, int nz, int zc, const float* __restrict__ r, float* __restrict__ x, const K125 K) {
+// CTA owns planes [z0, z0 + zc) of its 128 x 16 columns
+__global__ void __launch_bounds__(256, 2)
+    k_smoother_comp(int nx, int ny, int nz, int zc, const float* __restrict__ r, float* __restrict__ x,
+                    const __grid_constant__ K125x2 K) {
     constexpr int kPer = (kCompPlane + 255) / 256;  // staged elements per thread and plane
-    __shared__ __align__(16) float sp[2][kCompPlane];
+    __shared__ __align__(16) float sp[3][kCompPlane];
     const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
     const int x0 = blockIdx.x * kCompTX, y0 = blockIdx.y * kCompTY, z0 = blockIdx.z * zc;
     const int z1 = min(nz, z0 + zc);
-    const int ox = x0 + 4 * lx, oy = y0 + ly;  // first output of the thread
+    const int ox = x0 + 4 * lx, oy = y0 + 2 * ly;  // first output of the thread
     const int64_t plane = (int64_t)nx * ny;
-    const bool orow = oy < ny;
-    // the staged elements of this thread: offset within a plane, or -1 outside the box
-    int off[kPer];
+    // the staged elements of this thread: offset within a plane; outside the box
+    // the shared elements stay zero
+    unsigned off[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
         const int q = threadIdx.x + 256 * u;
-        const int c = q % kCompSX, rr = q / kCompSX;
+        // element q of the buffer: rows in pairs, (x, row 0), (x, row 1), with 16-byte
+        // pieces swapped in every second 128 bytes (see below)
+        const int e = q % (2 * kCompSX), pc = e >> 2, lc = pc ^ ((pc >> 3) & 1);
+        const int c = 2 * lc + ((e >> 1) & 1), rr = 2 * (q / (2 * kCompSX)) + (e & 1);
         const int gx = x0 - 2 + c, gy = y0 - 2 + rr;
-        off[u] = (q < kCompPlane && gx >= 0 && gx < nx && gy >= 0 && gy < ny) ? gy * nx + gx : -1;
+        off[u] = (q < kCompPlane && gx >= 0 && gx < nx && gy >= 0 && gy < ny) ? (unsigned)(gy * nx + gx) : ~0u;
+        if (q < kCompPlane && off[u] == ~0u) sp[0][q] = sp[1][q] = sp[2][q] = 0.f;
     }
-    float pre[kPer];
-    auto fetch = [&](int zr) {  // global loads of input plane zr into registers
+    const unsigned sbase = (unsigned)__cvta_generic_to_shared(&sp[0][threadIdx.x]);
+    auto fetch = [&](int zr, int buf) {  // input plane zr into a buffer
         const bool zin = zr >= 0 && zr < nz;
-        const float* rp = r + (int64_t)zr * plane;
+        const float* rp = r + (zin ? zr : 0) * plane;
+        const unsigned d = sbase + 4 * kCompPlane * buf;
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) pre[u] = (zin && off[u] >= 0) ? rp[off[u]] : 0.f;
+        for (int u = 0; u < kPer; ++u)
+            if (off[u] != ~0u) cp_async4_zfill(d + 1024 * u, rp + off[u], zin);
     };
-    auto put = [&](float* dst) {
+    // a thread reads 64 bytes of a row pair, 32 bytes after its neighbour's: with
+    // the swap eight lanes' 16-byte reads fall on all 32 banks
+    int po[4];
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int q = threadIdx.x + 256 * u;
-            if (q < kCompPlane) dst[q] = pre[u];
-        }
-    };
-    // acc[j][i]: output plane (input plane - 2 + j), x output ox + i
-    float acc[5][4];
+    for (int k = 0; k < 4; ++k) {
+        const int lc = 2 * lx + k;
+        po[k] = (ly * 2 * kCompSX) + 4 * (lc ^ ((lc >> 3) & 1));
+    }
+    // acc[j][i]: output plane (input plane - 2 + j), x output ox + i of rows oy (x) and oy + 1 (y)
+    float2 acc[5][4];
 #pragma unroll
     for (int j = 0; j < 5; ++j)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[j][i] = 0.f;
-    fetch(z0 - 2);
-    put(sp[0]);
-    fetch(z0 - 1);
-    __syncthreads();
+        for (int i = 0; i < 4; ++i) acc[j][i] = make_float2(0.f, 0.f);
+    fetch(z0 - 2, 0);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    fetch(z0 - 1, 1);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
     int buf = 0;
     for (int zi = z0 - 2; zi <= z1 + 1; ++zi) {
         // x of the output plane completed in this iteration, loaded now so that
         // the plane's multiply-adds hide the latency
         const int zo = zi - 2;
-        const bool ostore = zo >= z0 && zo < z1 && orow;
-        float xo[4];
+        const bool zst = zo >= z0 && zo < z1;
+        float xo[2][4];
         float* px = x + (int64_t)zo * plane + (int64_t)oy * nx + ox;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) xo[i] = (ostore && ox + i < nx) ? px[i] : 0.f;
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xo[v][i] = (zst && oy + v < ny && ox + i < nx) ? px[v * nx + i] : 0.f;
+        // plane zi has landed for every thread, and plane zi - 1 has been read by all:
+        // its buffer takes plane zi + 2
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();
+        if (zi + 2 <= z1 + 1) fetch(zi + 2, buf == 0 ? 2 : buf - 1);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
         // input plane zi feeds output planes zi - 2 .. zi + 2 (acc[0] .. acc[4]) with dz = 2 - j;
-        // output planes outside [z0, z1) are skipped (the same for the whole CTA)
-        bool need[5];
+        // those outside [z0, z1) are skipped (the same for the whole CTA, at its first and last
+        // planes; elsewhere no branch separates the five chains of multiply-adds)
+        float2 w[2][8];  // the row pair (row - 2, row - 1) from row oy, and the one after it
+        auto load = [&](float2(&d)[8], int pr) {
 #pragma unroll
-        for (int j = 0; j < 5; ++j) need[j] = zi - 2 + j >= z0 && zi - 2 + j < z1;
-        const float* p = sp[buf] + ly * kCompSX + 4 * lx;
-#pragma unroll
-        for (int dy = 0; dy < 5; ++dy) {
-            const float4 a = *reinterpret_cast<const float4*>(p + dy * kCompSX);
-            const float4 bq = *reinterpret_cast<const float4*>(p + dy * kCompSX + 4);
-            const float w[8] = {a.x, a.y, a.z, a.w, bq.x, bq.y, bq.z, bq.w};
-#pragma unroll
-            for (int j = 0; j < 5; ++j) {
-                if (!need[j]) continue;
-                const int dz = 2 - j;
-#pragma unroll
-                for (int dx = 0; dx < 5; ++dx) {
-                    const float kv = K.k[(dz + 2) * 25 + dy * 5 + dx];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(kv, w[i + dx], acc[j][i]);
-                }
+            for (int k = 0; k < 4; ++k) {
+                const float4 a = *reinterpret_cast<const float4*>(sp[buf] + po[k] + pr * 2 * kCompSX);
+                d[2 * k] = make_float2(a.x, a.y);
+                d[2 * k + 1] = make_float2(a.z, a.w);
             }
-        }
-        // output plane zi - 2 is complete
-        if (ostore) {
+        };
+        load(w[0], 0);
+        load(w[1], 1);
+        auto taps = [&](auto all) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (ox + i < nx) px[i] = xo[i] + acc[0][i];
+            for (int dy = 0; dy < 5; ++dy) {
+                float2 u[8];  // inputs of rows oy and oy + 1 at tap dy
+#pragma unroll
+                for (int q = 0; q < 8; ++q) u[q] = dy & 1 ? make_float2(w[0][q].y, w[1][q].x) : w[0][q];
+                if (dy == 1 || dy == 3) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) w[0][q] = w[1][q];
+                    if (dy == 1) load(w[1], 2);
+                }
+#pragma unroll
+                for (int dx = 0; dx < 5; ++dx)
+#pragma unroll
+                    for (int j = 0; j < 5; ++j) {
+                        if (!all.value && (zi - 2 + j < z0 || zi - 2 + j >= z1)) continue;
+                        const float2 kv = K.k[(4 - j) * 25 + dy * 5 + dx];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[j][i] = __ffma2_rn(kv, u[i + dx], acc[j][i]);
+                    }
+            }
+        };
+        if (zi - 2 >= z0 && zi + 2 < z1) taps(std::true_type{});
+        else taps(std::false_type{});
+        // output plane zi - 2 is complete
+        if (zst) {
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (oy + v < ny && ox + i < nx) px[v * nx + i] = xo[v][i] + (v ? acc[0][i].y : acc[0][i].x);
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[j][i] = acc[j + 1][i];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[4][i] = 0.f;
-        // plane zi + 1 (in registers) into the other buffer: its last readers
-        // (plane zi - 1) passed the previous barrier
-        if (zi + 1 <= z1 + 1) put(sp[buf ^ 1]);
-        __syncthreads();
-        if (zi + 2 <= z1 + 1) fetch(zi + 2);
-        buf ^= 1;
+        for (int i = 0; i < 4; ++i) acc[4][i] = make_float2(0.f, 0.f);
+        buf = buf == 2 ? 0 : buf + 1;
     }
 }
 
@@ -294,16 +336,16 @@ ew_status ComposedSmoother::build(const float* weights_dev, cudaStream_t st) {
 
 ew_status ComposedSmoother::apply(const GridGeom& g, const float* r, float* x, cudaStream_t st) const {
     if (g.dim != 3 || interior.size() != 125) return set_error(EW_EINVAL, "composed smoother: not built for a 3D grid");
-    K125 K;
-    std::memcpy(K.k, interior.data(), sizeof(K.k));
+    K125x2 K;
+    for (size_t q = 0; q < 125; ++q) K.k[q] = make_float2(interior[q], interior[q]);
     const int nx = (int)g.n[0], ny = (int)g.n[1], nz = (int)g.n[2];
-    // z chunks: as many as fill the resident CTA slots once (four a SM), at
+    // z chunks: as many as fill the resident CTA slots once (two a SM), at
     // least kCompZMin planes each (each chunk restages two planes on each side)
     int cdev = 0, nsm = 0;
     EW_CUDA_TRY(cudaGetDevice(&cdev));
     EW_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, cdev));
     const int bx = (nx + kCompTX - 1) / kCompTX, by = (ny + kCompTY - 1) / kCompTY;
-    const int nzc = std::max(1, (4 * nsm) / std::max(1, bx * by));
+    const int nzc = std::max(1, (2 * nsm) / std::max(1, bx * by));
     const int zc = std::max(std::min(kCompZMin, nz), (nz + nzc - 1) / nzc);
     dim3 grid((unsigned)bx, (unsigned)by, (unsigned)((nz + zc - 1) / zc));
     k_smoother_comp<<<grid, 256, 0, st>>>(nx, ny, nz, zc, r, x, K);
