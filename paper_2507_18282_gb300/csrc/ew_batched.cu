@@ -24,7 +24,7 @@
 #include <vector>
 
 #include "ew_internal.h"
-#include "ew_tb2d_dev.cuh"
+#include "ew_reg2d_dev.cuh"
 
 namespace ew {
 
@@ -61,6 +61,30 @@ __global__ void __launch_bounds__(32 * NWX * NTY, MINB)
     }
 }
 
+// the same rounds on tiles in registers (FP32)
+template <int R, int NW, int KY, int B, bool GEN>
+__global__ void __launch_bounds__(32 * NW, 1)
+    k_step_reg2d_batched(const BatchDesc<float>* __restrict__ descs, const BatchItem* __restrict__ items, int nitems) {
+    using S = Reg2dShape<R, NW, KY, B>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* stage = reinterpret_cast<float*>(smem_raw);
+    float* exch = stage + 3 * S::PLANE;
+    auto tile = [&](int it) {
+        const BatchItem w = items[it];
+        const BatchDesc<float>& d = descs[w.desc];
+        return Reg2dTile{d.nx, d.ny, d.st.bc, w.tile % d.ntx * S::TX - S::H, w.tile / d.ntx * S::TY - S::H,
+                         d.Ain, d.Bin, d.acc};
+    };
+    if ((int)blockIdx.x >= nitems) return;
+    reg2d_stage<R, NW, KY, B, GEN>(tile(blockIdx.x), stage);
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const BatchDesc<float>& d = descs[items[it].desc];
+        reg2d_steps<R, NW, KY, B, GEN>(tile(it), d.Aout, d.Bout, d.acc, d.cw, d.b, d.st, stage, exch, [&]() {
+            if (it + (int)gridDim.x < nitems) reg2d_stage<R, NW, KY, B, GEN>(tile(it + gridDim.x), stage);
+        });
+    }
+}
+
 struct BVariant {
     int B, TX, TY, threads;
     size_t smem;
@@ -75,13 +99,24 @@ struct BVariant {
             (void*)k_step_tb2d_batched<T, R, NWX, NTY, KY, B, MINB, true>                                \
     }
 
+#define EW_RVAR(R, NW, KY, B)                                                                              \
+    BVariant {                                                                                            \
+        B, Reg2dShape<R, NW, KY, B>::TX, Reg2dShape<R, NW, KY, B>::TY, Reg2dShape<R, NW, KY, B>::NT,      \
+            Reg2dShape<R, NW, KY, B>::SMEM, (void*)k_step_reg2d_batched<R, NW, KY, B, false>,             \
+            (void*)k_step_reg2d_batched<R, NW, KY, B, true>                                               \
+    }
+
+// 64 boxes of 255 to 2047 points a side, order 2: tiles in registers 16.0 ms
+// (depth 12) and 16.2 ms (depth 16), W in shared memory 20.5 ms at best (128 x 128
+// points, depth 16) and 21.1 ms (128 x 64, two CTAs an SM, depth 8: for batches of
+// few tiles).  At order 4 a point's rows no longer fit the registers at a useful
+// size: 32.5 ms against 31.5 ms, so those stay in shared memory.
 template <typename T, int R>
 static const std::vector<BVariant>& bvariants();
 template <>
 const std::vector<BVariant>& bvariants<float, 1>() {
-    static const std::vector<BVariant> v = {EW_BVAR(float, 1, 2, 8, 8, 4, 2),   EW_BVAR(float, 1, 2, 8, 8, 8, 2),
-                                            EW_BVAR(float, 1, 2, 16, 8, 8, 1),  EW_BVAR(float, 1, 2, 4, 16, 8, 2),
-                                            EW_BVAR(float, 1, 2, 16, 8, 12, 1), EW_BVAR(float, 1, 2, 16, 8, 16, 1)};
+    static const std::vector<BVariant> v = {EW_BVAR(float, 1, 2, 8, 8, 4, 2), EW_BVAR(float, 1, 2, 8, 8, 8, 2),
+                                            EW_RVAR(1, 12, 9, 12), EW_RVAR(1, 12, 9, 16)};
     return v;
 }
 template <>
@@ -330,7 +365,9 @@ static ew_status batched_t(std::vector<BProblem>& P, int order, cudaStream_t st,
     }
     int vi = 0;
     auto it = g_batch.tune.find(tkey);
-    if (variant_pin && *variant_pin >= 0 && *variant_pin < (int)vars.size()) {
+    if (const char* e = getenv("EW_BATCH_VARIANT")) {  // tuning and testing hook
+        vi = std::min(std::max(atoi(e), 0), (int)vars.size() - 1);
+    } else if (variant_pin && *variant_pin >= 0 && *variant_pin < (int)vars.size()) {
         vi = *variant_pin;
     } else if (it != g_batch.tune.end()) {
         vi = it->second;
