@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "ew_internal.h"
+#include "ew_small_eig.h"
 
 namespace ew {
 
@@ -48,7 +49,8 @@ ew_status filter_apply_any(ew_grid* g, const ew_filter_params* p, const FilterPl
 ew_status rayleigh_any(ew_grid* g, const void* phi, int nvec, double* lam, double* res, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// cyclic Jacobi for a small symmetric matrix (row-major n x n, destroyed).
+// cyclic Jacobi for a small symmetric matrix (row-major n x n, destroyed); the
+// Rayleigh-Ritz step's larger ones go to tridiagonal_eig (ew_small_eig.h).
 // Eigenvalues in w, eigenvectors in the columns of V (row-major).
 // ---------------------------------------------------------------------------
 void jacobi_eig(int n, std::vector<double>& A, std::vector<double>& V, std::vector<double>& w) {
@@ -356,7 +358,7 @@ struct KSRun {
         std::vector<double> A((size_t)n * n), Vv, w;
         for (int i = 0; i < n; ++i)
             for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = 0.5 * (h(i, j) + h(j, i));
-        jacobi_eig(n, A, Vv, w);
+        tridiagonal_eig(n, A, Vv, w);
         std::vector<int> ord(n);
         std::iota(ord.begin(), ord.end(), 0);
         std::sort(ord.begin(), ord.end(), [&](int a, int c) { return w[a] > w[c]; });
