@@ -473,7 +473,7 @@ def measure_cube3d(ew, flush, pk, pk_kind, steps, warmup):
     return dict(workload="cube3d_511_order2_fp32_explicit", metric=METRIC, unit=UNIT,
                 value=cells / (ms / 1e3) / 1e9, ms_per_step=ms / steps, steps=steps, warmup=warmup,
                 time_steps_per_step=info["Nt"], l2="flushed between timed steps (512 MB write)",
-                bound="hbm", kernel="k_step_tb3d<float, tuned depth>", bytes_per_launch=bytes_launch,
+                bound="hbm", kernel="k_step_tb3d_wide, tuned depth", bytes_per_launch=bytes_launch,
                 mean_launch_ms=mean, achieved=achieved, peak=float(pk["hbm_gbs"]), frac=achieved / float(pk["hbm_gbs"]),
                 peak_source=pk_kind,
                 # the profile covers the warm-up wave-solves too (each has the same launches)

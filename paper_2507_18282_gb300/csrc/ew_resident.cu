@@ -338,11 +338,11 @@ static int cluster_ctas(const GridGeom& g, int nvec) {
 }
 
 // The cluster form also takes larger grids with few vectors, which the blocked
-// kernels would run on a fraction of the SMs.  The line is where both took the
-// same time (400 steps): FP32 up to 4 x 255^2 points (order 4: 656 against
-// 1354 us; 16 x 181^2 1199 against 1358 us is left to the blocked form's
-// larger tiles); pairs 16 x 255^2 (3838 against 5781 us); FP64 4 x 255^2
-// (4830 against 4938 us), and 16 x 127^2 (3554 against 8124 us).
+// kernels would run on a fraction of the SMs.  The line is where the next form
+// takes the same time (400 steps): FP32 up to 181^2 points a vector (beyond, the
+// tiles of ew_persist2d.cu: 255^2, order 4, 455 against 597 us here); pairs 16 x
+// 255^2 (3838 against 5781 us blocked); FP64 4 x 255^2 (4830 against 4938 us
+// blocked), and 16 x 127^2 (3554 against 8124 us).
 template <typename T>
 static bool fits_cluster(const GridGeom& g, int nvec) {
     if (g.N > (sizeof(T) == 4 ? 32768 : 65536) || !cluster_ctas<T>(g, nvec)) return false;
