@@ -211,6 +211,10 @@ template <typename T>
 ew_status tb3d_advance(const GridGeom& g, const FilterPlan& plan, const T* cdev, T* const* F, int* prv, int* cur,
                        int64_t L, T* acc, int nvec, int64_t fstride, int tb, cudaStream_t st);
 
+// one launch of b <= B steps (B = 2, 3, 4) of its FP32 form on 32 x 32 regions
+ew_status tb3d_f2_step(int B, const GridGeom& g, const float* Din, const float* Win, float* Dout, float* Wout,
+                       float* acc, const float* cw, int b, const Stencil<float>& s, int nvec, int64_t fstride,
+                       cudaStream_t st);
 // the FP32 form for both orders (ew_tb3d_wide.cu)
 bool tb3d_wide_fits(const GridGeom& g, int nvec);
 ew_status tb3d_wide_tune(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,

@@ -411,6 +411,23 @@ static ew_status launch_depth(int b, const GridGeom& g, const float* Din, const 
 #undef EW_W
 }
 
+// Second order, kNarrow + depth: the 32 x 32 regions of ew_tb3d.cu.  They can win
+// where the 64 x 32 regions overhang the box by a fifth or more or the planes are
+// few (27 x 463 x 132 3.0 against 3.8 ms, 374 x 122 x 30 374 against 390 us), so
+// there the tuner times them too; without the tuner (a depth asked for) they take
+// the boxes up to 32 points wide.
+constexpr int kNarrow = 16;
+static bool narrow_may_win(const GridGeom& g) {
+    const double over = (double)((g.n[0] + 59) / 60 * 60) / g.n[0] * ((g.n[1] + 27) / 28 * 28) / g.n[1];
+    return g.order == 2 && (over > 1.2 || g.n[2] < 64);
+}
+static ew_status launch_variant(int v, int b, const GridGeom& g, const float* Din, const float* Win, float* Dout,
+                                float* Wout, float* acc, const float* cw, const Stencil<float>& s, int nvec,
+                                int64_t fstride, cudaStream_t st) {
+    if (v >= kNarrow) return tb3d_f2_step(v - kNarrow, g, Din, Win, Dout, Wout, acc, cw, b, s, nvec, fstride, st);
+    return launch_depth(b, g, Din, Win, Dout, Wout, acc, cw, s, nvec, fstride, st);
+}
+
 // depth autotuner (second order): times depths 2..4 on the caller's buffers
 // (before the real wave-solve overwrites them) and caches the fastest per grid
 // shape.  Fourth order: depth 2 (a rim of 4; depth 3 would leave 20 of 32 rows)
@@ -434,10 +451,12 @@ ew_status tb3d_wide_tune(const GridGeom& g, const FilterPlan& plan, const float*
     EW_TRY(ev.create());
     int best = 3;
     double best_rate = -1.0;
-    for (int B = 2; B <= 4; ++B) {
+    for (int v : {2, 3, 4, kNarrow + 2, kNarrow + 3, kNarrow + 4}) {
+        const int B = v % kNarrow;
+        if (v >= kNarrow && !narrow_may_win(g)) continue;
         for (int rep = 0; rep < 3; ++rep) {  // one warm launch, two timed
             if (rep == 1) EW_CUDA_TRY(cudaEventRecord(ev.a, st));
-            EW_TRY(launch_depth(B, g, F[0], F[1], F[2], F[3], acc, cdev, s, nvec, fstride, st));
+            EW_TRY(launch_variant(v, B, g, F[0], F[1], F[2], F[3], acc, cdev, s, nvec, fstride, st));
         }
         EW_CUDA_TRY(cudaEventRecord(ev.b, st));
         EW_CUDA_TRY(cudaEventSynchronize(ev.b));
@@ -445,11 +464,11 @@ ew_status tb3d_wide_tune(const GridGeom& g, const FilterPlan& plan, const float*
         EW_CUDA_TRY(cudaEventElapsedTime(&ms, ev.a, ev.b));
         const double rate = 2.0 * B / std::max(ms, 1e-6f);  // time steps per ms
         if (getenv("EW_TUNE_LOG"))
-            fprintf(stderr, "[ew tune] %lldx%lldx%lld 3D order 2 fp32: depth %d: %.4f ms/step\n", (long long)g.n[0],
-                    (long long)g.n[1], (long long)g.n[2], B, 1.0 / rate);
+            fprintf(stderr, "[ew tune] %lldx%lldx%lld 3D order 2 fp32: depth %d%s: %.4f ms/step\n", (long long)g.n[0],
+                    (long long)g.n[1], (long long)g.n[2], B, v >= kNarrow ? ", 32 x 32" : "", 1.0 / rate);
         if (rate > best_rate) {
             best_rate = rate;
-            best = B;
+            best = v;
         }
     }
     std::lock_guard<std::mutex> lk(g_tb3w_mu);
@@ -473,12 +492,19 @@ ew_status tb3d_wide_advance(const GridGeom& g, const FilterPlan& plan, const flo
         auto it = g_tb3w_cache.find(Tb3dKey{g.n[0], g.n[1], g.n[2], nvec, dev});
         if (it != g_tb3w_cache.end()) B = it->second;
     }
+    int v = 0;  // variant: below kNarrow the 64 x 32 regions
+    if (B >= kNarrow) {
+        v = B;
+        B -= kNarrow;
+    } else if (tb > 1 && g.order == 2 && g.n[0] <= 32) {
+        v = kNarrow + B;
+    }
     int p = *prv, c = *cur, a = -1, d = -1;
     for (int q = 0; q < 4; ++q)
         if (q != p && q != c) (a < 0 ? a : d) = q;
     while (L < plan.Nt) {
         const int b = (int)std::min<int64_t>(B, plan.Nt - L);
-        EW_TRY(launch_depth(b, g, F[p], F[c], F[a], F[d], acc, cdev + L + 1, s, nvec, fstride, st));
+        EW_TRY(launch_variant(v, b, g, F[p], F[c], F[a], F[d], acc, cdev + L + 1, s, nvec, fstride, st));
         L += b;
         std::swap(p, a);
         std::swap(c, d);
