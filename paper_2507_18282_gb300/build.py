@@ -44,7 +44,8 @@ def _stale(obj: str, src: str, headers) -> bool:
 def build(verbose: bool = False, jobs: int | None = None) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
-    headers = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+    headers = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    headers += glob.glob(os.path.join(HERE, "..", "include", "*.h"))
     srcs = sources()
     objs = []
     todo = []
