@@ -488,12 +488,9 @@ struct MGSolver {
     int nsm = 0, pl_occ[2] = {1, 1};  // SMs; resident plane-kernel CTAs a SM (order 2, order 4)
     bool f2 = false;                  // FP32: the paired form (ew_mg_plane.cu)
     template <int MODE>
-    void plane3d(const GridGeom& g_, const T* x, const T* b, T* out, const Stencil<T>& sa, T wd, int colour) {
+    ew_status plane3d(const GridGeom& g_, const T* x, const T* b, T* out, const Stencil<T>& sa, T wd, int colour) {
         if constexpr (sizeof(T) == 4)
-            if (f2) {
-                mg_plane3d_f2(MODE, g_, x, b, out, sa, wd, colour, nsm, st);
-                return;
-            }
+            if (f2) return mg_plane3d_f2(MODE, g_, x, b, out, sa, wd, colour, nsm, st);
         const int nx = (int)g_.n[0], ny = (int)g_.n[1], nz = (int)g_.n[2];
         const int bx = (nx + kPlBX - 1) / kPlBX, by = (ny + kPlBY - 1) / kPlBY;
         // z chunks: enough CTAs to fill the resident slots once, at least 8 planes each
@@ -506,16 +503,18 @@ struct MGSolver {
         else
             k_mg_plane3d<T, 4, MODE><<<grid, kPlNT, PlaneRing<T, 4>::SMEM, st>>>(nx, ny, nz, zc, x, b, out, sa, wd,
                                                                               colour);
+        EW_CUDA_TRY(cudaGetLastError());
         count_launch();
+        return EW_OK;
     }
-    void resid(int L, const Stencil<T>& sa) { plane3d<0>(lv[L], X[L], B[L], R[L], sa, T(0), 0); }
+    ew_status resid(int L, const Stencil<T>& sa) { return plane3d<0>(lv[L], X[L], B[L], R[L], sa, T(0), 0); }
 
     // 3D levels
     ew_status smooth(int L, int steps) {
         Stencil<T> sa = make_stencil<T>(lv[L], a);
         for (int s = 0; s < steps; ++s) {
             if (L < p->learned_levels) {
-                resid(L, sa);
+                EW_TRY(resid(L, sa));
                 if constexpr (sizeof(T) == 4) {
                     if (use_comp) {
                         EW_TRY(comp[L].apply(lv[L], R[L], X[L], st));
@@ -527,9 +526,9 @@ struct MGSolver {
                 // 3D levels: one launch per colour
                 const int ncol = lv[L].order == 2 ? 2 : 3;
                 for (int colour = 0; colour < ncol; ++colour)
-                    plane3d<2>(lv[L], X[L], B[L], X[L], sa, weight(L, sa), colour);
+                    EW_TRY(plane3d<2>(lv[L], X[L], B[L], X[L], sa, weight(L, sa), colour));
             } else {
-                plane3d<1>(lv[L], X[L], B[L], Tm[L], sa, weight(L, sa), 0);
+                EW_TRY(plane3d<1>(lv[L], X[L], B[L], Tm[L], sa, weight(L, sa), 0));
                 std::swap(X[L], Tm[L]);
             }
         }
@@ -623,7 +622,7 @@ struct MGSolver {
             return mg_prolong2d<T>(f, c, X[L + 1], X[L], st);
         }
         EW_TRY(smooth(L, p->pre));
-        resid(L, sa);
+        EW_TRY(resid(L, sa));
         k_mg_restrict3d<T><<<pt_grid(c.n[0], c.n[1], c.n[2]), pt_threads(c.n[0]), 0, st>>>(
             f.n[0], f.n[1], f.n[2], c.n[0], c.n[1], c.n[2], R[L], B[L + 1], X[L + 1]);
         count_launch();
@@ -659,7 +658,7 @@ struct MGSolver {
             EW_TRY(mg_resid_norm2d<T>(lv[0], X[0], B[0], make_stencil<T>(lv[0], a), dpart, nb, st));
             EW_TRY(launch_finish_sum(dpart, nb, 1, dres, st));
         } else {
-            resid(0, make_stencil<T>(lv[0], a));
+            EW_TRY(resid(0, make_stencil<T>(lv[0], a)));
             EW_TRY(launch_dots<T>(R[0], R[0], lv[0].N, 1, dpart, dres, st));
         }
         void* hp = nullptr;  // page-locked: a copy into pageable memory is staged by the driver
@@ -821,9 +820,9 @@ ew_status mg_collect_residuals(ew_grid* g, double a, const ew_mg_params* mp, int
         for (int c = 0; c < 3 && k < nsamples && s == EW_OK; ++c) {
             float* r = out + (size_t)k * N;
             const GridGeom& gg = g->geom;
-            mg.template plane3d<0>(gg, mg.X[0], mg.B[0], r, sa, 0.f, 0);
+            s = mg.template plane3d<0>(gg, mg.X[0], mg.B[0], r, sa, 0.f, 0);
             ++k;
-            s = mg.vcycle(0);
+            if (s == EW_OK) s = mg.vcycle(0);
         }
     }
     cudaStreamSynchronize(st);

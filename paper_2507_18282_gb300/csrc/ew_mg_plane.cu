@@ -16,6 +16,8 @@
 // of the cycles).  Measured, 255^3 order 4, one residual: 90 us (64 x 8 columns a
 // CTA, scalar instructions, every stencil point from shared memory) -> 79 us;
 // Jacobi sweep on 31^3 10.0 -> 6.6 us.
+#include <stdlib.h>
+
 #include <algorithm>
 
 #include "ew_internal.h"
@@ -235,6 +237,8 @@ static ew_status plane(const GridGeom& g, const float* x, const float* b, float*
 
 ew_status mg_plane3d_f2(int mode, const GridGeom& g, const float* x, const float* b, float* out,
                         const Stencil<float>& sa, float wd, int colour, int nsm, cudaStream_t st) {
+    if (const char* e = getenv("EW_TEST_MG_PLANE_FAIL"))  // test hook: launches of this mode fail
+        if (atoi(e) == mode) return cuda_error(cudaErrorLaunchOutOfResources, "multigrid plane kernel (test hook)");
     if (mode == 0) return plane<0>(g, x, b, out, sa, wd, colour, nsm, st);
     if (mode == 1) return plane<1>(g, x, b, out, sa, wd, colour, nsm, st);
     return plane<2>(g, x, b, out, sa, wd, colour, nsm, st);
