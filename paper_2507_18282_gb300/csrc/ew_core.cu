@@ -214,17 +214,19 @@ ew_status pinned(ew_grid* g, size_t bytes, void** out) {
     return EW_OK;
 }
 
-// upload the filter weights (type T) into the grid's misc scratch
+// upload the filter weights (type T) into the grid's misc scratch, with zeros after
+// them: the tuners time each candidate's full depth from the table's start, which may
+// be more steps than a short solve has
 template <typename T>
 static ew_status upload_weights(ew_grid* g, const FilterPlan& plan, cudaStream_t st, const T** out) {
-    size_t n = plan.c.size();
+    const size_t nc = plan.c.size(), n = nc + kMaxDepth;
     EW_TRY(g->misc.reserve(n * sizeof(T)));
     void* hp = nullptr;
     EW_TRY(pinned(g, n * sizeof(T), &hp));
     // the pinned buffer may still feed an earlier copy on this stream
     EW_CUDA_TRY(cudaStreamSynchronize(st));
     T* h = (T*)hp;
-    for (size_t i = 0; i < n; ++i) h[i] = (T)plan.c[i];
+    for (size_t i = 0; i < n; ++i) h[i] = i < nc ? (T)plan.c[i] : T(0);
     EW_CUDA_TRY(cudaMemcpyAsync(g->misc.ptr, h, n * sizeof(T), cudaMemcpyHostToDevice, st));
     *out = (const T*)g->misc.ptr;
     return EW_OK;

@@ -252,6 +252,10 @@ ew_status tma2d_launch(const Tma2dDesc& d, const GridGeom& g, const float* Ain, 
 // reads (and clears) the flag a staging wait of the TMA-staged step sets when it gives up
 ew_status tma2d_check_timeout();
 
+// the most time steps a candidate of the tuners takes in one launch: the device
+// table of filter weights holds that many entries after the solve's own
+constexpr int kMaxDepth = 32;
+
 // distance between consecutive vectors of a wave-solve's time-level fields:
 // N rounded up to 64 points, so every vector starts on a 256-byte boundary
 // (bulk copies need 16-byte aligned rows)

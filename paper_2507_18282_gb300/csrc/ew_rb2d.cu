@@ -53,6 +53,7 @@ struct Rb2dShape {
     static constexpr size_t XBUF_BYTES = 2 * (size_t)NTY * 2 * R * 32 * sizeof(float4);
     static constexpr size_t SMEM = STAGE_BYTES + XBUF_BYTES + 16;  // + the mbarrier
     static_assert(TX > 0 && TY > 0, "rim larger than the tile");
+    static_assert(B <= kMaxDepth, "the tuner times B steps on any solve's weights");
 };
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }

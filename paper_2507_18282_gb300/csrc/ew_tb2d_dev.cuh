@@ -79,6 +79,7 @@ struct Tb2dShape {
     static constexpr int NT = 32 * NWX * NTY;
     static constexpr size_t SMEM = sizeof(T) * 2 * (size_t)PX * RY;
     static_assert(TX > 0 && TY > 0, "halo larger than the tile");
+    static_assert(B <= kMaxDepth, "the tuner times B steps on any solve's weights");
 };
 
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
