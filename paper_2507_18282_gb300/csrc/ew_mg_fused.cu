@@ -10,8 +10,12 @@
 //   k_mg_bottom             the rest of the cycle from a small level down to
 //                           the coarsest and back, one launch of one CTA
 //
-// Each takes the operations of the elementary kernels in their order, point by
-// point, so a cycle gives the same bits whichever form its levels take.
+// A sweep, a residual and a restriction take the operations of one elementary
+// kernel a point in their order, whichever form a level takes.  Two things differ
+// between the forms, by rounding: the prolongation adds the four coarse values in
+// pairs in k_mg_smooth2d and one by one in k_mg_bottom, and the coarsest level is
+// solved by sine transforms in k_mg_bottom (up to kMgSineMax points an axis) but by
+// conjugate gradients in a launch of its own (k_mg_coarse_cg).
 #include <math.h>
 
 #include <algorithm>
@@ -66,14 +70,13 @@ __global__ void k_mg_prolong2d(int nx, int ny, int cx, int cy, const T* __restri
 // fourth-order stencil's point beyond a wall is the negated mirror, which is
 // the point itself at the wall's neighbour.
 //
-// FP64 levels are bound by the FP64 units (two operations a clock and SM), so
-// they take the update with its constants folded: x + w (b - M x) =
-// k0 x + w b + sum k_i (neighbour sums), k0 = 1 - w (1 - c0) (0 for the colour
-// sweeps), k_i = w c_i, with w b staged once: 4-5 operations a point and sweep
-// instead of 8.  (The rounding of w and k_i biases a sweep by about an ulp of
-// x; the residual that the next level and the stopping test see is still that
-// of the stored stencil.  FP32 levels keep the residual form: there an ulp
-// matters and the FP32 units do not.)
+// FP64 levels are bound by the FP64 units (two operations a clock and SM): eight
+// operations a point and sweep.  The update stays in the residual form all the
+// same: with its constants multiplied out (k0 x + w b + sum w c_i (neighbour
+// sums), four or five operations) a sweep rounds differently from the residual
+// that the stopping test sees, and the lowest ||b - M x|| / ||b|| that a solve
+// reaches rises by up to 2.9 times (order 4, colour sweeps, 255^2; 1.4 and 2.0 on
+// 1023^2 at order 2).
 // Why: at 1023^2 in FP64 a V(2,2) cycle issued 88 launches of 2-16 us; the
 // halo costs 20 % more points at TILE 32 (two red-black sweeps), 42 % at 16.
 template <typename T, int ORDER, bool GS, int NS, int TILE>
@@ -91,7 +94,6 @@ __global__ void __launch_bounds__(256)
                   T wd, const T* __restrict__ ec, int cx, int cy) {
     using S = Smooth2dShape<T, ORDER, GS, NS, TILE>;
     constexpr int R = S::R, H = S::H, SX = S::SX, SB = S::SB, NC = S::NC, P = S::P;
-    constexpr bool FOLD = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem_ms[];
     T* cur = reinterpret_cast<T*>(smem_ms);
     T* nxt = GS ? cur : cur + SX * SX;
@@ -134,12 +136,8 @@ __global__ void __launch_bounds__(256)
     for (int q = tid; q < SB * SB; q += 256) {
         const int sy = q / SB, sx = q - sy * SB;
         const int gx = x0 - (H - R) + sx, gy = y0 - (H - R) + sy;
-        const T v = (gx >= 0 && gx < nx && gy >= 0 && gy < ny) ? b[(int64_t)gy * nx + gx] : T(0);
-        sb[q] = FOLD ? m_mul(wd, v) : v;
+        sb[q] = (gx >= 0 && gx < nx && gy >= 0 && gy < ny) ? b[(int64_t)gy * nx + gx] : T(0);
     }
-    // folded constants
-    const T k0 = T(1) - wd * (T(1) - sa.c0);
-    const T k1x = wd * sa.c1[0], k1y = wd * sa.c1[1], k2x = wd * sa.c2[0], k2y = wd * sa.c2[1];
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < P; ++p) {
@@ -171,21 +169,14 @@ __global__ void __launch_bounds__(256)
                 s2x = m_add(xl, xh);
                 s2y = m_add(yl, yh);
             }
-            if (FOLD) {
-                T v = GS ? bv : m_fma(k0, u, bv);
-                v = m_fma(k1y, s1y, m_fma(k1x, s1x, v));
-                if (ORDER == 4) v = m_fma(k2y, s2y, m_fma(k2x, s2x, v));
-                nxt[c] = v;
-            } else {
-                T lap = m_mul(sa.c0, u);
-                lap = m_fma(sa.c1[0], s1x, lap);
-                lap = m_fma(sa.c1[1], s1y, lap);
-                if (ORDER == 4) {
-                    lap = m_fma(sa.c2[0], s2x, lap);
-                    lap = m_fma(sa.c2[1], s2y, lap);
-                }
-                nxt[c] = m_fma(wd, m_add(m_add(bv, -u), lap), u);
+            T lap = m_mul(sa.c0, u);
+            lap = m_fma(sa.c1[0], s1x, lap);
+            lap = m_fma(sa.c1[1], s1y, lap);
+            if (ORDER == 4) {
+                lap = m_fma(sa.c2[0], s2x, lap);
+                lap = m_fma(sa.c2[1], s2y, lap);
             }
+            nxt[c] = m_fma(wd, m_add(m_add(bv, -u), lap), u);
         }
         __syncthreads();
         if (!GS) {
@@ -360,23 +351,9 @@ __global__ void __launch_bounds__(kBotThreads) k_mg_bottom(const MgBottom<T> m) 
         const T* b = base + off[l] + 2 * N;
         const Stencil<T> sa = L.sa;
         const T wd = L.wd;
-        // FP64: x + wd (b - M x) with folded constants, as in k_mg_smooth2d
-        Stencil<T> sf = sa;
-        if (sizeof(T) == 8)
-            for (int d = 0; d < 3; ++d) {
-                sf.c1[d] *= wd;
-                sf.c2[d] *= wd;
-            }
-        const T k0 = T(1) - wd * (T(1) - sa.c0);
         auto update = [&](const T* x, int q, int i, int j, int k) {
-            if constexpr (sizeof(T) == 8) {
-                T v = wd * b[q];
-                if (!m.colours) v += k0 * x[q];
-                return bsum<T, DIM, ORDER>(x, sf, v, q, i, j, k, nx, ny, nz);
-            } else {
-                const T u = x[q];
-                return u + wd * ((b[q] - u) + bsum<T, DIM, ORDER>(x, sa, sa.c0 * u, q, i, j, k, nx, ny, nz));
-            }
+            const T u = x[q];
+            return u + wd * ((b[q] - u) + bsum<T, DIM, ORDER>(x, sa, sa.c0 * u, q, i, j, k, nx, ny, nz));
         };
         for (int s = 0; s < steps; ++s) {
             T* x = X(l);
