@@ -275,17 +275,26 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
                               cudaStream_t st);
 
 // --- whole wave-solve of a small 2D grid on chip (ew_resident.cu) ------------
+struct ResidentPlan {
+    int C = 0;             // CTAs a vector; 0: the grid does not take this path
+    void* kern = nullptr;  // the cluster form's kernel (NULL: the one-CTA form)
+    int PT = 0;            // points a thread
+    int pts = 0;           // points of the fullest CTA
+    int threads = 0;
+    bool blocked = false;  // the operations of the blocked kernels
+    size_t smem = 0;
+};
 template <typename T>
-bool resident_fits(const GridGeom& g, int nvec);
+ResidentPlan resident_plan(const GridGeom& g, int nvec);
 template <typename T>
-ew_status resident_wave_solve(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
-                              cudaStream_t st);
+ew_status resident_wave_solve(const GridGeom& g, const ResidentPlan& p, const T* vin, T* vout, const T* cw,
+                              const FilterPlan& plan, int nvec, cudaStream_t st);
 
 // --- 2D wave-solves that fit on the chip, one cooperative launch (ew_persist2d.cu)
 bool persist2d_fits(const GridGeom& g, int nvec);
 size_t persist2d_room(const GridGeom& g, int nvec);  // bytes it needs after the time-level fields
 ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
-                            int nvec, int64_t fstride, void* records, cudaStream_t st);
+                            int nvec, int64_t fstride, void* records, cudaStream_t st, bool* taken);
 // reads (and clears) the flag a halo exchange sets when it gives up
 ew_status persist2d_check_timeout();
 

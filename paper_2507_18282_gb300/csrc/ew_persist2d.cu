@@ -380,9 +380,12 @@ size_t persist2d_room(const GridGeom& g, int nvec) {
     return sizeof(unsigned long long) * 4 * (size_t)g.N * (size_t)nvec;
 }
 
-// steps 2 .. Nt: F[0] = D^1, F[1] = W^1 (dense rows), acc holds c_0 W^0 + c_1 W^1
+// steps 2 .. Nt: F[0] = D^1, F[1] = W^1 (dense rows), acc holds c_0 W^0 + c_1 W^1.
+// *taken = false when the device refuses the launch because its CTAs cannot all be
+// resident (a partitioned GPU): nothing was computed and the caller takes the blocked kernels.
 ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
-                            int nvec, int64_t fstride, void* records, cudaStream_t st) {
+                            int nvec, int64_t fstride, void* records, cudaStream_t st, bool* taken) {
+    *taken = true;
     if (plan.Nt < 2) return EW_OK;
     const PersistPlan p = persist_plan(g, nvec, sm_count());
     if (!p.v) return set_error(EW_EUNSUPPORTED, "grid does not fit on the chip");
@@ -397,8 +400,17 @@ ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const flo
     void* args[] = {(void*)&nx, (void*)&ny, (void*)&D1,  (void*)&W1,  (void*)&acc,     (void*)&cdev, (void*)&Nt,
                     (void*)&s,  (void*)&ntx, (void*)&nty, (void*)&fstride, (void*)&rec,  (void*)&stall};
     cudaEvent_t ev = fused_begin(st);
-    EW_CUDA_TRY(cudaLaunchCooperativeKernel(p.v->fn, dim3((unsigned)(ntx * nty * nvec)), dim3((unsigned)p.v->threads),
-                                            args, p.v->smem, st));
+    cudaError_t e = getenv("EW_TEST_COOP_TOO_LARGE")  // test hook: the answer of a device with fewer SMs
+                        ? cudaErrorCooperativeLaunchTooLarge
+                        : cudaLaunchCooperativeKernel(p.v->fn, dim3((unsigned)(ntx * nty * nvec)),
+                                                      dim3((unsigned)p.v->threads), args, p.v->smem, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        if (ev) cudaEventDestroy(ev);
+        *taken = false;
+        return EW_OK;
+    }
+    EW_CUDA_TRY(e);
     fused_end(ev, st, g.N * nvec, g.N * nvec * (plan.Nt - 1));
     return EW_OK;
 }

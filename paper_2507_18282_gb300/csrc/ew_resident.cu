@@ -345,19 +345,85 @@ static int cluster_ctas(const GridGeom& g, int nvec) {
 // blocked), and 16 x 127^2 (3554 against 8124 us).
 template <typename T>
 static bool fits_cluster(const GridGeom& g, int nvec) {
-    if (g.N > (sizeof(T) == 4 ? 32768 : 65536) || !cluster_ctas<T>(g, nvec)) return false;
+    if (g.N > (sizeof(T) == 4 ? 32768 : 65536)) return false;
     if (std::is_same<T, dd>::value) return nvec <= 16;
     if (g.N * nvec > 262144 + 2048) return false;
     return sizeof(T) == 4 || g.N <= 16384 || nvec <= 4;
 }
 
-template <typename T>
-bool resident_fits(const GridGeom& g, int nvec) {
-    return g.dim == 2 && !g.map && (fits_cta<T>(g, nvec) || fits_cluster<T>(g, nvec));
+template <typename T, int R, bool BLOCKED>
+static void* cluster_kernel(int PT) {
+    if (PT == 1) return (void*)k_resident2d_cluster<T, R, 1, BLOCKED>;
+    return PT == 2 ? (void*)k_resident2d_cluster<T, R, 2, BLOCKED> : (void*)k_resident2d_cluster<T, R, 4, BLOCKED>;
 }
-template bool resident_fits<float>(const GridGeom&, int);
-template bool resident_fits<double>(const GridGeom&, int);
-template bool resident_fits<dd>(const GridGeom&, int);
+
+// the launch of the cluster form with C CTAs a vector
+template <typename T>
+static ResidentPlan cluster_plan(const GridGeom& g, bool blocked, int C) {
+    ResidentPlan p;
+    // points a thread: 512 threads beat 1024 once each has two points (a barrier of fewer warps;
+    // 127^2 FP32 order 4, 16 CTAs, 8 vectors, 400 steps: 565 us with one point, 365 with two, 408 with four)
+    p.pts = (int)((g.n[1] + C - 1) / C * g.n[0]);  // points of the fullest CTA
+    p.PT = p.pts <= 512 ? 1 : p.pts <= 1024 ? 2 : 4;
+    p.C = C;
+    p.blocked = blocked;
+    p.threads = ((p.pts + p.PT - 1) / p.PT + 31) / 32 * 32;
+    p.smem = 2 * sizeof(T) * (size_t)((g.n[1] + C - 1) / C + 4) * (size_t)(g.n[0] + 4);
+    if (g.order == 2)
+        p.kern = blocked ? cluster_kernel<T, 1, true>(p.PT) : cluster_kernel<T, 1, false>(p.PT);
+    else
+        p.kern = blocked ? cluster_kernel<T, 2, true>(p.PT) : cluster_kernel<T, 2, false>(p.PT);
+    return p;
+}
+
+static cudaLaunchConfig_t cluster_config(const ResidentPlan& p, int nvec, cudaLaunchAttribute* at, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(nvec * p.C));
+    cfg.blockDim = dim3((unsigned)p.threads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)p.C;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// One cluster of this plan can be resident: 16 CTAs are beyond the portable size, and where fewer SMs of a
+// GPC are visible (a partitioned GPU) less than that may be too many.  The query takes 0.2 us.
+static bool cluster_fits_device(const ResidentPlan& p) {
+    if (const char* e = getenv("EW_TEST_MAX_CLUSTER"))  // test hook: no larger clusters on this device
+        if (p.C > atoi(e)) return false;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(p, 1, &at, nullptr);
+    int n = 0;
+    if (cudaFuncSetAttribute(p.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) == cudaSuccess &&
+        cudaFuncSetAttribute(p.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, p.kern, &cfg) == cudaSuccess)
+        return n > 0;
+    cudaGetLastError();
+    return false;
+}
+
+template <typename T>
+ResidentPlan resident_plan(const GridGeom& g, int nvec) {
+    if (g.dim != 2 || g.map) return ResidentPlan();
+    const bool cta = fits_cta<T>(g, nvec);
+    if (cta || fits_cluster<T>(g, nvec))
+        // smaller clusters where the wanted ones do not fit the device, as far as their CTAs' points allow
+        for (int C = cluster_ctas<T>(g, nvec); C > 0; C /= 2) {
+            const ResidentPlan p = cluster_plan<T>(g, !cta, C);
+            if (p.pts > kResMaxPts || (std::is_same<T, double>::value && C == 1)) break;
+            if (cluster_fits_device(p)) return p;
+        }
+    ResidentPlan one;
+    if (cta) one.C = 1, one.pts = (int)g.N;
+    return one;
+}
+template ResidentPlan resident_plan<float>(const GridGeom&, int);
+template ResidentPlan resident_plan<double>(const GridGeom&, int);
+template ResidentPlan resident_plan<dd>(const GridGeom&, int);
 
 // one-CTA form
 template <typename T, int R>
@@ -371,69 +437,32 @@ static ew_status resident_cta(const GridGeom& g, const T* vin, T* vout, const T*
     return EW_OK;
 }
 
-template <typename T, int R, int PT, bool BLOCKED>
-static ew_status resident_cluster_pt(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan,
-                                     int nvec, int C, int threads, const Stencil<T>& s, const Stencil<T>& sh,
-                                     cudaStream_t st) {
-    const size_t smem = 2 * sizeof(T) * (size_t)((g.n[1] + C - 1) / C + 4) * (size_t)(g.n[0] + 4);
-    auto kern = k_resident2d_cluster<T, R, PT, BLOCKED>;
-    EW_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    EW_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(nvec * C));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    EW_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (int)g.n[0], (int)g.n[1], vin, vout, cw, plan.Nt, s, sh));
-    return EW_OK;
-}
-
-template <typename T, int R, bool BLOCKED>
-static ew_status resident_cluster(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan,
-                                  int nvec, int C, const Stencil<T>& s, const Stencil<T>& sh, cudaStream_t st) {
-    // points a thread: 512 threads beat 1024 once each has two points (a barrier of fewer warps;
-    // 127^2 FP32 order 4, 16 CTAs, 8 vectors, 400 steps: 565 us with one point, 365 with two, 408 with four)
-    const int64_t pts = (g.n[1] + C - 1) / C * g.n[0];  // points of the fullest CTA
-    const int PT = pts <= 512 ? 1 : pts <= 1024 ? 2 : 4;
-    const int threads = (int)(((pts + PT - 1) / PT + 31) / 32 * 32);
-    if (PT == 1) return resident_cluster_pt<T, R, 1, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
-    if (PT == 2) return resident_cluster_pt<T, R, 2, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
-    return resident_cluster_pt<T, R, 4, BLOCKED>(g, vin, vout, cw, plan, nvec, C, threads, s, sh, st);
-}
-
-template <typename T, int R>
-static ew_status resident_r(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
-                            cudaStream_t st) {
-    const Stencil<T> s = make_stencil<T>(g, plan.dt * plan.dt);
-    const Stencil<T> sh = make_stencil<T>(g, 0.5 * plan.dt * plan.dt);
-    const int C = cluster_ctas<T>(g, nvec);
-    if (!fits_cta<T>(g, nvec)) return resident_cluster<T, R, true>(g, vin, vout, cw, plan, nvec, C, s, sh, st);
-    if (C > 0) return resident_cluster<T, R, false>(g, vin, vout, cw, plan, nvec, C, s, sh, st);
-    return resident_cta<T, R>(g, vin, vout, cw, plan, nvec, s, sh, st);
-}
-
 template <typename T>
-ew_status resident_wave_solve(const GridGeom& g, const T* vin, T* vout, const T* cw, const FilterPlan& plan, int nvec,
-                              cudaStream_t st) {
+ew_status resident_wave_solve(const GridGeom& g, const ResidentPlan& p, const T* vin, T* vout, const T* cw,
+                              const FilterPlan& plan, int nvec, cudaStream_t st) {
+    Stencil<T> s = make_stencil<T>(g, plan.dt * plan.dt);
+    Stencil<T> sh = make_stencil<T>(g, 0.5 * plan.dt * plan.dt);
     cudaEvent_t ev = fused_begin(st);
-    if (g.order == 2)
-        EW_TRY((resident_r<T, 1>(g, vin, vout, cw, plan, nvec, st)));
-    else
-        EW_TRY((resident_r<T, 2>(g, vin, vout, cw, plan, nvec, st)));
+    if (p.kern) {
+        int nx = (int)g.n[0], ny = (int)g.n[1];
+        int64_t Nt = plan.Nt;
+        void* args[] = {(void*)&nx, (void*)&ny, (void*)&vin, (void*)&vout, (void*)&cw, (void*)&Nt, (void*)&s, (void*)&sh};
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = cluster_config(p, nvec, &at, st);
+        EW_CUDA_TRY(cudaLaunchKernelExC(&cfg, p.kern, args));
+    } else if (g.order == 2) {
+        EW_TRY((resident_cta<T, 1>(g, vin, vout, cw, plan, nvec, s, sh, st)));
+    } else {
+        EW_TRY((resident_cta<T, 2>(g, vin, vout, cw, plan, nvec, s, sh, st)));
+    }
     fused_end(ev, st, g.N * nvec, g.N * nvec * plan.Nt);
     return EW_OK;
 }
-template ew_status resident_wave_solve<float>(const GridGeom&, const float*, float*, const float*, const FilterPlan&,
-                                              int, cudaStream_t);
-template ew_status resident_wave_solve<double>(const GridGeom&, const double*, double*, const double*,
-                                               const FilterPlan&, int, cudaStream_t);
-template ew_status resident_wave_solve<dd>(const GridGeom&, const dd*, dd*, const dd*, const FilterPlan&, int,
-                                           cudaStream_t);
+template ew_status resident_wave_solve<float>(const GridGeom&, const ResidentPlan&, const float*, float*, const float*,
+                                              const FilterPlan&, int, cudaStream_t);
+template ew_status resident_wave_solve<double>(const GridGeom&, const ResidentPlan&, const double*, double*,
+                                               const double*, const FilterPlan&, int, cudaStream_t);
+template ew_status resident_wave_solve<dd>(const GridGeom&, const ResidentPlan&, const dd*, dd*, const dd*,
+                                           const FilterPlan&, int, cudaStream_t);
 
 }  // namespace ew

@@ -323,17 +323,21 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
     }
     // the variant override EW_TB2D_VARIANT (a tuning and testing hook) selects a
     // blocked kernel, so it also bypasses the on-chip path of small grids
-    if (temporal_block == 0 && resident_fits<T>(g, nvec) && !getenv("EW_TB2D_VARIANT"))
-        return resident_wave_solve<T>(g, vin, vout, cdev, plan, nvec, st);
+    if (temporal_block == 0 && !getenv("EW_TB2D_VARIANT")) {
+        const ResidentPlan rp = resident_plan<T>(g, nvec);
+        if (rp.C > 0) return resident_wave_solve<T>(g, rp, vin, vout, cdev, plan, nvec, st);
+    }
     // fields are laid out [field][vector][point]; 2D rows may be padded (pitch2d)
     const int64_t fstride = wave_field_stride(g);
     T* F[4];
     for (int q = 0; q < 4; ++q) F[q] = fields + (int64_t)q * nvec * fstride;
     if constexpr (std::is_same<T, float>::value)
         if (temporal_block == 0 && persist2d_fits(g, nvec) && !getenv("EW_TB2D_VARIANT")) {
+            bool taken = true;
             EW_TRY(first_step<T>(g, vin, F[0], F[1], vout, plan, nvec, fstride, st, g.n[0]));
-            return persist2d_advance(g, plan, cdev, F, vout, nvec, fstride,
-                                     fields + 4 * (int64_t)nvec * fstride, st);
+            EW_TRY(persist2d_advance(g, plan, cdev, F, vout, nvec, fstride, fields + 4 * (int64_t)nvec * fstride, st,
+                                     &taken));
+            if (taken) return EW_OK;
         }
     const bool blocked = g.dim == 2 && temporal_block != 1;
     // the tuner writes the spare fields and the filter sum, so it runs before the first step
