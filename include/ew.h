@@ -484,8 +484,12 @@ ew_status ew_smoother_train(const ew_grid* grid, double half_dt2, const ew_train
  * benchmarks): the kernel's name with its template shape, NUL-terminated in
  * name_host (cap bytes), the time steps per launch (*depth) and the owned
  * tile of a CTA (*tile_x x *tile_y points); depth and tiles may be NULL.
- * EW_EINVAL when no wave-solve of this shape has been tuned in this process,
- * or for a grid other than a 2D box.  Host only. */
+ * Where the last wave-solve of this shape ran on the chip in one launch
+ * instead, the on-chip kernel, the time steps between two exchanges of its
+ * CTAs and the points of its fullest CTA.
+ * EW_EINVAL when no wave-solve of this shape has been tuned or run so in this
+ * process (grids that one CTA holds are never tuned), or for a grid other than
+ * a 2D box.  Host only. */
 ew_status ew_tuned_variant(const ew_grid* grid, int nvec, char* name_host, int cap, int* depth, int* tile_x,
                            int* tile_y);
 

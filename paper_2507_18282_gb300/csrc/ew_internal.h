@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <functional>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -274,6 +275,17 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
                               const T* vin, T* vout, int nvec, T* fields, int temporal_block,
                               cudaStream_t st);
 
+// What ew_tuned_variant reports of a shape that was solved on the chip in place of
+// the blocked kernels: the kernel with its template shape, the steps between two
+// exchanges of its CTAs, the points of the fullest CTA.  `id` tells forms of a shape
+// apart; `describe` runs only when the shape's form is new.
+struct OnChipForm {
+    std::string kernel;
+    int depth, TX, TY;
+};
+template <typename T>
+void tb2d_note_on_chip(const GridGeom& g, int nvec, const void* id, const std::function<OnChipForm()>& describe);
+
 // --- whole wave-solve of a small 2D grid on chip (ew_resident.cu) ------------
 struct ResidentPlan {
     int C = 0;             // CTAs a vector; 0: the grid does not take this path
@@ -287,11 +299,14 @@ struct ResidentPlan {
 template <typename T>
 ResidentPlan resident_plan(const GridGeom& g, int nvec);
 template <typename T>
+OnChipForm resident_form(const GridGeom& g, const ResidentPlan& p);
+template <typename T>
 ew_status resident_wave_solve(const GridGeom& g, const ResidentPlan& p, const T* vin, T* vout, const T* cw,
                               const FilterPlan& plan, int nvec, cudaStream_t st);
 
 // --- 2D wave-solves that fit on the chip, one cooperative launch (ew_persist2d.cu)
 bool persist2d_fits(const GridGeom& g, int nvec);
+OnChipForm persist2d_form(const GridGeom& g, int nvec);
 size_t persist2d_room(const GridGeom& g, int nvec);  // bytes it needs after the time-level fields
 ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
                             int nvec, int64_t fstride, void* records, cudaStream_t st, bool* taken);

@@ -308,12 +308,14 @@ struct PersistVariant {
     int R, TX, TY, H, threads, per_sm;
     size_t smem;
     double us[2];  // time of a step with one and with two CTAs an SM
+    const char* name;
 };
 #define EW_PERSIST(R, NWX, NTY, KY, B, MINB, US1, US2)                                                               \
     PersistVariant {                                                                                                \
         (void*)k_persist2d<R, NWX, NTY, KY, B, MINB>, R, PersistShape<R, NWX, NTY, KY, B>::TX,                      \
             PersistShape<R, NWX, NTY, KY, B>::TY, PersistShape<R, NWX, NTY, KY, B>::H,                              \
-            PersistShape<R, NWX, NTY, KY, B>::NT, MINB, PersistShape<R, NWX, NTY, KY, B>::SMEM, { US1, US2 }        \
+            PersistShape<R, NWX, NTY, KY, B>::NT, MINB, PersistShape<R, NWX, NTY, KY, B>::SMEM, { US1, US2 },       \
+            "k_persist2d<" #R ", " #NWX ", " #NTY ", " #KY ", " #B ", " #MINB ">"                                    \
     }
 // Times measured over 400 steps, exchanges included.  A step's time is mostly
 // latency (a region of 64 x 32 points takes 0.6 us, 128 x 64 points 1.4 us), so
@@ -373,6 +375,12 @@ static int sm_count() {
 bool persist2d_fits(const GridGeom& g, int nvec) {
     if (g.dim != 2 || g.map) return false;
     return persist_plan(g, nvec, sm_count()).us <= (g.order == 2 ? 2.05 : 3.2);
+}
+
+OnChipForm persist2d_form(const GridGeom& g, int nvec) {
+    const PersistPlan p = persist_plan(g, nvec, sm_count());
+    if (!p.v) return OnChipForm{"", 0, 0, 0};
+    return OnChipForm{p.v->name, p.v->H / p.v->R, (int)((g.n[0] + p.ntx - 1) / p.ntx), (int)((g.n[1] + p.nty - 1) / p.nty)};
 }
 
 // bytes of the exchange records, which follow the time-level fields

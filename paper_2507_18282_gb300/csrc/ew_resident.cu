@@ -5,6 +5,7 @@
 // launch (eqs. explicitStep1, explicitScheme, filterQuadrature; the summed
 // form of ew_stencil.cu).
 #include <cooperative_groups.h>
+#include <stdio.h>
 #include <stdlib.h>
 
 #include <algorithm>
@@ -436,6 +437,18 @@ static ew_status resident_cta(const GridGeom& g, const T* vin, T* vout, const T*
     EW_CUDA_TRY(cudaGetLastError());
     return EW_OK;
 }
+
+template <typename T>
+OnChipForm resident_form(const GridGeom& g, const ResidentPlan& p) {
+    char buf[96];
+    snprintf(buf, sizeof buf, "k_resident2d_cluster<%s, %d, %d, %s>",
+             sizeof(T) == 4 ? "float" : std::is_same<T, dd>::value ? "dd" : "double", g.order == 2 ? 1 : 2, p.PT,
+             p.blocked ? "true" : "false");
+    return OnChipForm{buf, 1, (int)g.n[0], (int)((g.n[1] + p.C - 1) / p.C)};
+}
+template OnChipForm resident_form<float>(const GridGeom&, const ResidentPlan&);
+template OnChipForm resident_form<double>(const GridGeom&, const ResidentPlan&);
+template OnChipForm resident_form<dd>(const GridGeom&, const ResidentPlan&);
 
 template <typename T>
 ew_status resident_wave_solve(const GridGeom& g, const ResidentPlan& p, const T* vin, T* vout, const T* cw,

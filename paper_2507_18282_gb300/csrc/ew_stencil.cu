@@ -325,7 +325,11 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
     // blocked kernel, so it also bypasses the on-chip path of small grids
     if (temporal_block == 0 && !getenv("EW_TB2D_VARIANT")) {
         const ResidentPlan rp = resident_plan<T>(g, nvec);
-        if (rp.C > 0) return resident_wave_solve<T>(g, rp, vin, vout, cdev, plan, nvec, st);
+        if (rp.C > 0) {
+            EW_TRY(resident_wave_solve<T>(g, rp, vin, vout, cdev, plan, nvec, st));
+            if (rp.blocked) tb2d_note_on_chip<T>(g, nvec, rp.kern, [&]() { return resident_form<T>(g, rp); });
+            return EW_OK;
+        }
     }
     // fields are laid out [field][vector][point]; 2D rows may be padded (pitch2d)
     const int64_t fstride = wave_field_stride(g);
@@ -337,7 +341,10 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
             EW_TRY(first_step<T>(g, vin, F[0], F[1], vout, plan, nvec, fstride, st, g.n[0]));
             EW_TRY(persist2d_advance(g, plan, cdev, F, vout, nvec, fstride, fields + 4 * (int64_t)nvec * fstride, st,
                                      &taken));
-            if (taken) return EW_OK;
+            if (taken) {
+                tb2d_note_on_chip<T>(g, nvec, (const void*)persist2d_fits, [&]() { return persist2d_form(g, nvec); });
+                return EW_OK;
+            }
         }
     const bool blocked = g.dim == 2 && temporal_block != 1;
     // the tuner writes the spare fields and the filter sum, so it runs before the first step

@@ -313,11 +313,16 @@ static ew_status autotune(const GridGeom& g, T* const* F, T* acc, const T* cw, c
 }
 
 template <typename T>
+static void forget_on_chip(const GridGeom& g, int nvec);
+
+template <typename T>
 ew_status tb2d_tune(const GridGeom& g, const FilterPlan& plan, const T* cdev, T* const* F, T* acc, int nvec,
                     int64_t fstride, cudaStream_t st) {
     Stencil<T> s = make_stencil<T>(g, plan.dt * plan.dt);
     int vi = 0;
-    return autotune<T>(g, F, acc, cdev, s, nvec, fstride, st, &vi, false);
+    EW_TRY(autotune<T>(g, F, acc, cdev, s, nvec, fstride, st, &vi, false));
+    forget_on_chip<T>(g, nvec);  // this solve runs on the blocked kernels
+    return EW_OK;
 }
 template ew_status tb2d_tune<float>(const GridGeom&, const FilterPlan&, const float*, float* const*, float*, int,
                                     int64_t, cudaStream_t);
@@ -385,6 +390,52 @@ template int64_t tb2d_field_pitch<double>(const GridGeom&, const FilterPlan&, co
 template int64_t tb2d_field_pitch<dd>(const GridGeom&, const FilterPlan&, const dd*, dd* const*, dd*, int, int64_t,
                                       int, cudaStream_t);
 
+// shapes solved on the chip (a mixture of faces may take different forms)
+struct OnChipNote {
+    const void* id;
+    OnChipForm form;
+};
+static std::map<std::pair<TuneKey, int>, OnChipNote> g_on_chip;  // guarded by g_tune_mu
+
+template <typename T>
+static std::pair<TuneKey, int> on_chip_key(const GridGeom& g, int nvec) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return {TuneKey{g.n[0], g.n[1], g.order, MantBits<T>::value, nvec, dev}, g.bc};
+}
+template <typename T>
+void tb2d_note_on_chip(const GridGeom& g, int nvec, const void* id, const std::function<OnChipForm()>& describe) {
+    const auto key = on_chip_key<T>(g, nvec);
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    const auto it = g_on_chip.find(key);
+    if (it == g_on_chip.end() || it->second.id != id) g_on_chip[key] = OnChipNote{id, describe()};
+}
+template void tb2d_note_on_chip<float>(const GridGeom&, int, const void*, const std::function<OnChipForm()>&);
+template void tb2d_note_on_chip<double>(const GridGeom&, int, const void*, const std::function<OnChipForm()>&);
+template void tb2d_note_on_chip<dd>(const GridGeom&, int, const void*, const std::function<OnChipForm()>&);
+
+template <typename T>
+static void forget_on_chip(const GridGeom& g, int nvec) {
+    const auto key = on_chip_key<T>(g, nvec);
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_on_chip.erase(key);
+}
+
+// the on-chip form of the shape's last solve, if it ran on the chip
+template <typename T>
+static bool on_chip_choice(const GridGeom& g, int nvec, std::string* name, int* B, int* TX, int* TY) {
+    const auto key = on_chip_key<T>(g, nvec);
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    const auto it = g_on_chip.find(key);
+    if (it == g_on_chip.end()) return false;
+    const OnChipForm& f = it->second.form;
+    *name = f.kernel;
+    *B = f.depth;
+    *TX = f.TX;
+    *TY = f.TY;
+    return true;
+}
+
 // description of the tuned choice (for reports)
 template <typename T>
 int tb2d_choice(const GridGeom& g, int nvec, int* B, int* TX, int* TY) {
@@ -434,16 +485,21 @@ extern "C" ew_status ew_tuned_variant(const ew_grid* grid, int nvec, char* name_
     if (g.dim != 2 || g.map) return set_error(EW_EINVAL, "not a 2D box grid");
     int B = 0, TX = 0, TY = 0, vi = -1;
     std::string name;
-    if (grid->prec == EW_FP32) {
-        vi = tb2d_choice<float>(g, nvec, &B, &TX, &TY);
-        if (vi >= 0) name = tb2d_choice_name<float>(g, vi);
-    } else if (grid->prec == EW_FP64) {
-        vi = tb2d_choice<double>(g, nvec, &B, &TX, &TY);
-        if (vi >= 0) name = tb2d_choice_name<double>(g, vi);
-    } else {
-        vi = tb2d_choice<dd>(g, nvec, &B, &TX, &TY);
-        if (vi >= 0) name = tb2d_choice_name<dd>(g, vi);
-    }
+    auto look = [&](auto t) {
+        using T = decltype(t);
+        if (on_chip_choice<T>(g, nvec, &name, &B, &TX, &TY)) {
+            vi = 0;
+            return;
+        }
+        vi = tb2d_choice<T>(g, nvec, &B, &TX, &TY);
+        if (vi >= 0) name = tb2d_choice_name<T>(g, vi);
+    };
+    if (grid->prec == EW_FP32)
+        look(float());
+    else if (grid->prec == EW_FP64)
+        look(double());
+    else
+        look(dd());
     if (vi < 0) return set_error(EW_EINVAL, "no wave-solve of this grid shape and nvec has been tuned");
     snprintf(name_host, (size_t)cap, "%s", name.c_str());
     if (depth) *depth = B;
