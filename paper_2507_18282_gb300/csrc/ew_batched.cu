@@ -109,14 +109,21 @@ struct BVariant {
 // 64 boxes of 255 to 2047 points a side, order 2: tiles in registers 16.0 ms
 // (depth 12) and 16.2 ms (depth 16), W in shared memory 20.5 ms at best (128 x 128
 // points, depth 16) and 21.1 ms (128 x 64, two CTAs an SM, depth 8: for batches of
-// few tiles).  At order 4 a point's rows no longer fit the registers at a useful
+// few tiles).  The tile of 128 x 128 points at depth 16 stays because its 98 x 98
+// owned points fit some batches better: 16 boxes of 255 x 260, 40 steps each, 158
+// us against 175 us on the register tiles, 53 of 457 x 85 588 against 619 us.
+// (160 random batches, 2 to 80 boxes of 40 to 1535 points a side: 159 are fastest
+// on the register tiles; depths 8 and 12 of 128 x 128 points and 64 x 128 points at
+// depth 8 were never fastest.)
+// At order 4 a point's rows no longer fit the registers at a useful
 // size: 32.5 ms against 31.5 ms, so those stay in shared memory.
 template <typename T, int R>
 static const std::vector<BVariant>& bvariants();
 template <>
 const std::vector<BVariant>& bvariants<float, 1>() {
     static const std::vector<BVariant> v = {EW_BVAR(float, 1, 2, 8, 8, 4, 2), EW_BVAR(float, 1, 2, 8, 8, 8, 2),
-                                            EW_RVAR(1, 12, 9, 12), EW_RVAR(1, 12, 9, 16)};
+                                            EW_RVAR(1, 12, 9, 12), EW_RVAR(1, 12, 9, 16),
+                                            EW_BVAR(float, 1, 2, 16, 8, 16, 1)};
     return v;
 }
 template <>
