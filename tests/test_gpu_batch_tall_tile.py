@@ -31,6 +31,7 @@ def test_candidate_and_bits(monkeypatch, capfd, bc):
     monkeypatch.delenv("EW_TUNE_LOG")
     for q, g in enumerate(grids):
         out = torch.empty_like(vin[q])
+        params[q].temporal_block = 2  # the blocked kernels, also for boxes that one CTA holds
         ew.ew_filter_apply(g, params[q], vin[q], out)
         torch.cuda.synchronize()
         assert torch.equal(out, vout[q]), boxes[q]
