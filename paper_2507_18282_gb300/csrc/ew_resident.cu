@@ -343,10 +343,13 @@ static int cluster_ctas(const GridGeom& g, int nvec) {
 // takes the same time (400 steps): FP32 up to 181^2 points a vector (beyond, the
 // tiles of ew_persist2d.cu: 255^2, order 4, 455 against 597 us here); pairs 16 x
 // 255^2 (3838 against 5781 us blocked); FP64 4 x 255^2 (4830 against 4938 us
-// blocked), and 16 x 127^2 (3554 against 8124 us).
+// blocked), and 16 x 127^2 (3554 against 8124 us).  FP64 at order 4 crosses at
+// 61,000 points (40 steps: 200^2 468 against 684 us blocked, 62,664 points 703
+// against 688, 256^2 709 against 688).
 template <typename T>
 static bool fits_cluster(const GridGeom& g, int nvec) {
     if (g.N > (sizeof(T) == 4 ? 32768 : 65536)) return false;
+    if (std::is_same<T, double>::value && g.order == 4 && g.N > 60000) return false;
     if (std::is_same<T, dd>::value) return nvec <= 16;
     if (g.N * nvec > 262144 + 2048) return false;
     return sizeof(T) == 4 || g.N <= 16384 || nvec <= 4;
@@ -391,20 +394,49 @@ static cudaLaunchConfig_t cluster_config(const ResidentPlan& p, int nvec, cudaLa
     return cfg;
 }
 
-// One cluster of this plan can be resident: 16 CTAs are beyond the portable size, and where fewer SMs of a
-// GPC are visible (a partitioned GPU) less than that may be too many.  The query takes 0.2 us.
-static bool cluster_fits_device(const ResidentPlan& p) {
+// Clusters of this plan that the device holds at a time.  16 CTAs are beyond the portable size, and where
+// fewer SMs of a GPC are visible (a partitioned GPU) less than that may be too many: 0.  The query takes 0.2 us.
+static int clusters_at_a_time(const ResidentPlan& p) {
     if (const char* e = getenv("EW_TEST_MAX_CLUSTER"))  // test hook: no larger clusters on this device
-        if (p.C > atoi(e)) return false;
+        if (p.C > atoi(e)) return 0;
     cudaLaunchAttribute at;
     const cudaLaunchConfig_t cfg = cluster_config(p, 1, &at, nullptr);
     int n = 0;
     if (cudaFuncSetAttribute(p.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) == cudaSuccess &&
         cudaFuncSetAttribute(p.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&n, p.kern, &cfg) == cudaSuccess)
-        return n > 0;
+        return n;
     cudaGetLastError();
-    return false;
+    return 0;
+}
+
+// Many vectors of a grid too large for one CTA of the cluster form: its clusters
+// and the one-CTA form (152 vectors a wave) then differ by how full their last
+// waves are.  One CTA takes 2.6 + 1.35e-4 N times as long for a vector as a CTA of
+// four in FP32 (N = 8200: 262 against 282 us for 152 vectors of 55 x 149, order 2, 60
+// steps; 1026 against 1144 us for 608 of 57 x 144, order 4), which loses where the
+// waves come out no longer: (24 x 500, 176 vectors: 472 against 252 us); at order 4
+// narrow grids (28 columns and fewer) and more than 9500 points stay with the
+// clusters (18 x 508, 140 vectors: 306 against 258 us).  Pairs in clusters of two:
+// only a second wave of a few CTAs loses (264 x 17, 77 vectors, order 2: 269 against
+// 282 us).
+template <typename T>
+static bool one_cta_wins(const GridGeom& g, int nvec, int C) {
+    if (nvec <= 76) return false;
+    if (std::is_same<T, dd>::value) return C == 2 && nvec * C > 152 && nvec * C <= 172;
+    if (sizeof(T) != 4 || C != 4 || (g.order == 4 && (g.n[0] < 32 || g.N > 9500))) return false;
+    return (nvec * C + 151) / 152 > (nvec + 151) / 152 * (2.6 + 1.35e-4 * (double)g.N);
+}
+
+// Pairs at order 4 where the clusters take several waves: a wave takes 1.4 + 0.8e-3
+// pts us a step (pts: points a CTA), the blocked kernels 9.2 us up to about 664,000
+// points of all vectors where their tiles fill (444 x 91, 40 steps: 14 vectors, two
+// waves, 297 against 367 us; 15 vectors, three waves, 425 against 374 us; but 59 x
+// 593, 16 vectors, 282 against 569 us)
+static bool pairs_blocked_wins(const GridGeom& g, int nvec, const ResidentPlan& p, int at_a_time) {
+    const int waves = (nvec + at_a_time - 1) / at_a_time;
+    return g.order == 4 && waves > 1 && g.N * nvec <= 664000 && p.pts >= 2550 && g.n[0] >= 100 &&
+           waves * (1.4 + 0.8e-3 * p.pts) > 9.2;
 }
 
 template <typename T>
@@ -416,7 +448,11 @@ ResidentPlan resident_plan(const GridGeom& g, int nvec) {
         for (int C = cluster_ctas<T>(g, nvec); C > 0; C /= 2) {
             const ResidentPlan p = cluster_plan<T>(g, !cta, C);
             if (p.pts > kResMaxPts || (std::is_same<T, double>::value && C == 1)) break;
-            if (cluster_fits_device(p)) return p;
+            if (cta && one_cta_wins<T>(g, nvec, C)) break;
+            const int n = clusters_at_a_time(p);
+            if (n == 0) continue;
+            if (!cta && std::is_same<T, dd>::value && pairs_blocked_wins(g, nvec, p, n)) break;
+            return p;
         }
     ResidentPlan one;
     if (cta) one.C = 1, one.pts = (int)g.N;
