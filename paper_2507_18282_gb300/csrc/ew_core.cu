@@ -242,7 +242,7 @@ static ew_status filter_apply_t(ew_grid* g, const ew_filter_params* p, const Fil
     const T* cdev = nullptr;
     EW_TRY(upload_weights<T>(g, plan, st, &cdev));
     size_t room = (size_t)4 * nvec * wave_field_stride(g->geom) * sizeof(T);
-    if (sizeof(T) == 4 && p->temporal_block == 0 && persist2d_fits(g->geom, nvec)) room += persist2d_room(g->geom, nvec);
+    if (sizeof(T) == 4 && p->temporal_block == 0 && persist2d_fits(g->geom, nvec, plan.Nt)) room += persist2d_room(g->geom, nvec);
     EW_TRY(g->fields.reserve(room));
     return explicit_wave_solve<T>(g->geom, plan, cdev, vin, vout, nvec, (T*)g->fields.ptr, p->temporal_block, st);
 }

@@ -305,7 +305,7 @@ ew_status resident_wave_solve(const GridGeom& g, const ResidentPlan& p, const T*
                               const FilterPlan& plan, int nvec, cudaStream_t st);
 
 // --- 2D wave-solves that fit on the chip, one cooperative launch (ew_persist2d.cu)
-bool persist2d_fits(const GridGeom& g, int nvec);
+bool persist2d_fits(const GridGeom& g, int nvec, int64_t Nt);
 OnChipForm persist2d_form(const GridGeom& g, int nvec);
 size_t persist2d_room(const GridGeom& g, int nvec);  // bytes it needs after the time-level fields
 ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,

@@ -368,13 +368,18 @@ static int sm_count() {
     return nsm;
 }
 
-// All vectors of the call fit the chip at once, and a step is faster than a
-// step of the blocked kernels, whose time does not fall below 3.25 us (order
-// 4) or 2.05 us (order 2) however small the grid (measured 300 x 250 ... 1000 x
-// 700; at 1023^2 with one vector both forms take 3.3 us, order 4).
-bool persist2d_fits(const GridGeom& g, int nvec) {
+// All vectors of the call fit the chip at once, and the solve is faster than on
+// the blocked kernels, whose step does not fall below 3.3 us (order 4; 3.7 us with
+// Neumann faces) or 2.8 us (order 2) however small the grid (measured 300 x 250 ...
+// 1600 x 700).  The largest order-4 regions take 3.12 us a step and 25 us a solve, so
+// with Dirichlet faces they pay only from about 200 steps (blocked against here: 446 x
+// 754, 4 vectors, 40 steps 155 and 164 us; 422 x 1364, 2 vectors, 100 steps 334 and 348
+// us; 1657 x 700, 240 steps 821 and 809 us; with a Neumann face 340 x 567, 6 vectors,
+// 100 steps 441 and 356 us).
+bool persist2d_fits(const GridGeom& g, int nvec, int64_t Nt) {
     if (g.dim != 2 || g.map) return false;
-    return persist_plan(g, nvec, sm_count()).us <= (g.order == 2 ? 2.05 : 3.2);
+    const double most = g.order == 2 ? 2.05 : g.bc != 0 || Nt >= 200 ? 3.2 : 3.0;
+    return persist_plan(g, nvec, sm_count()).us <= most;
 }
 
 OnChipForm persist2d_form(const GridGeom& g, int nvec) {

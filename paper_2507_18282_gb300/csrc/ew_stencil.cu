@@ -336,7 +336,7 @@ ew_status explicit_wave_solve(const GridGeom& g, const FilterPlan& plan, const T
     T* F[4];
     for (int q = 0; q < 4; ++q) F[q] = fields + (int64_t)q * nvec * fstride;
     if constexpr (std::is_same<T, float>::value)
-        if (temporal_block == 0 && persist2d_fits(g, nvec) && !getenv("EW_TB2D_VARIANT")) {
+        if (temporal_block == 0 && persist2d_fits(g, nvec, plan.Nt) && !getenv("EW_TB2D_VARIANT")) {
             bool taken = true;
             EW_TRY(first_step<T>(g, vin, F[0], F[1], vout, plan, nvec, fstride, st, g.n[0]));
             EW_TRY(persist2d_advance(g, plan, cdev, F, vout, nvec, fstride, fields + 4 * (int64_t)nvec * fstride, st,

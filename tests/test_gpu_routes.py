@@ -34,3 +34,10 @@ def _solve(n, order, prec, nvec, bc, spp):
     ((444, 91), 4, "fp32x2", 15, "k_step_tb2d"), ((59, 593), 4, "fp32x2", 16, "k_resident2d_cluster")])
 def test_cluster_or_blocked(n, order, prec, nvec, kernel):
     assert _solve(n, order, prec, nvec, "DDDD", 20).startswith(kernel)
+
+
+@pytest.mark.parametrize("n,nvec,bc,spp,kernel", [
+    ((446, 754), 4, "DDDD", 40, "k_step_"), ((446, 754), 4, "DDDD", 200, "k_persist2d"),
+    ((446, 752), 4, "NDDD", 40, "k_persist2d"), ((268, 425), 6, "DDDD", 40, "k_persist2d")])
+def test_cooperative_or_blocked(n, nvec, bc, spp, kernel):
+    assert _solve(n, 4, "fp32", nvec, bc, spp).startswith(kernel)
