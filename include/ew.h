@@ -33,8 +33,10 @@
  *    a failed host allocation inside a call returns EW_ENOMEM.
  *    Device-side waits are bounded and report EW_ETIMEOUT.  A wave-solve
  *    returns before its kernels run, so a wait that gave up there is reported
- *    by the next call that synchronises (the autotuner, ew_rayleigh and the
- *    solvers built on it); the outputs of that wave-solve are then invalid.
+ *    once, by the next call that synchronises (the autotuner, ew_rayleigh and
+ *    the solvers built on it) on the same grid handle, or on any handle from
+ *    the thread that launched the wave-solve; the outputs of that wave-solve
+ *    are then invalid.
  */
 #ifndef EW_H_
 #define EW_H_

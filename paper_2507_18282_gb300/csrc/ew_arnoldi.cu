@@ -841,6 +841,7 @@ ew_status arnoldi_eigs_impl(const ew_grid* grid, const ew_filter_params* params,
         EW_CUDA_TRY(cudaMemcpyAsync(vecs_dev, final_vecs, sizeof(double) * (size_t)ks.N * nw,
                                     cudaMemcpyDeviceToDevice, st));
     EW_CUDA_TRY(cudaStreamSynchronize(st));
+    EW_TRY(check_gave_up(g->geom));  // filter applications that another thread launched for this solver (hook)
     r.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (rep) *rep = r;
     return status;

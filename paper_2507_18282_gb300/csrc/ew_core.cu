@@ -214,6 +214,52 @@ ew_status pinned(ew_grid* g, size_t bytes, void** out) {
     return EW_OK;
 }
 
+// flags of the grids that the thread launched solves on; a destroyed grid's is kept until the next look
+static thread_local std::vector<std::shared_ptr<WaitFlag>> t_armed;
+static thread_local bool t_gave_up = false;  // found set on a destroyed grid
+static int thread_number() {
+    static std::atomic<int> count{0};
+    static thread_local const int mine = ++count;
+    return mine;
+}
+
+ew_status arm_gave_up(ew_grid* g) {
+    if (!g->gave_up) {
+        auto f = std::make_shared<WaitFlag>();
+        EW_CUDA_TRY(cudaMallocHost((void**)&f->p, sizeof(int)));
+        *f->p = 0;
+        g->gave_up = f;
+        g->geom.gave_up = f->p;
+    }
+    g->gave_up->thread = thread_number();
+    for (size_t i = 0; i < t_armed.size();) {
+        if (t_armed[i] == g->gave_up) return EW_OK;
+        if (t_armed[i].use_count() == 1) {  // its grid is gone, and with it its solves
+            t_gave_up = t_gave_up || (t_armed[i]->thread == thread_number() && *(volatile int*)t_armed[i]->p);
+            t_armed.erase(t_armed.begin() + (long)i);
+        } else {
+            ++i;
+        }
+    }
+    t_armed.push_back(g->gave_up);
+    return EW_OK;
+}
+
+ew_status check_gave_up(const GridGeom& g) {
+    bool hit = t_gave_up;
+    t_gave_up = false;
+    auto take = [&](int* p) {
+        if (p && *(volatile int*)p) {
+            *(volatile int*)p = 0;
+            hit = true;
+        }
+    };
+    take(g.gave_up);
+    for (auto& f : t_armed)
+        if (f->thread == thread_number()) take(f->p);
+    return hit ? set_error(EW_ETIMEOUT, "a bounded wait of a wave-solve (staging copy or halo exchange) gave up") : EW_OK;
+}
+
 // upload the filter weights (type T) into the grid's misc scratch, with zeros after
 // them: the tuners time each candidate's full depth from the table's start, which may
 // be more steps than a short solve has
@@ -240,6 +286,7 @@ static ew_status filter_apply_t(ew_grid* g, const ew_filter_params* p, const Fil
                                 T* vout, int nvec, cudaStream_t st) {
     if (p->scheme == EW_IMPLICIT) return implicit_wave_solve_any(g, plan, p, vin, vout, nvec, st);
     const T* cdev = nullptr;
+    if (sizeof(T) == 4) EW_TRY(arm_gave_up(g));  // only FP32 steps have kernels that wait
     EW_TRY(upload_weights<T>(g, plan, st, &cdev));
     size_t room = (size_t)4 * nvec * wave_field_stride(g->geom) * sizeof(T);
     if (sizeof(T) == 4 && p->temporal_block == 0 && persist2d_fits(g->geom, nvec, plan.Nt)) room += persist2d_room(g->geom, nvec);
@@ -498,10 +545,7 @@ static ew_status rayleigh_t(ew_grid* g, const T* phi, int nvec, double* lam_host
     double* h = (double*)hp;
     EW_CUDA_TRY(cudaMemcpyAsync(h, dnum, sizeof(double) * 2 * nvec, cudaMemcpyDeviceToHost, st));
     EW_CUDA_TRY(cudaStreamSynchronize(st));
-    EW_TRY(rb2d_check_timeout());  // a register-blocked wave-solve before this point gave up a wait
-    EW_TRY(tma2d_check_timeout());  // the same for a TMA-staged one
-    EW_TRY(persist2d_check_timeout());
-    if (g->geom.map) EW_TRY(mapped_check_timeout());
+    EW_TRY(check_gave_up(g->geom));
     std::vector<double> lam2(nvec);
     for (int j = 0; j < nvec; ++j) {
         double den = h[nvec + j];

@@ -6,6 +6,7 @@
 
 #include <atomic>
 #include <functional>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -135,6 +136,7 @@ struct GridGeom {
     double h[3];
     int64_t N;     // active points
     int bc = 0;    // face mask, as in Stencil
+    int* gave_up = nullptr;  // page-locked word that a kernel's bounded wait sets when it gives up (WaitFlag; may be NULL)
     MappedData* map = nullptr;  // a curvilinear grid (2D, order 2, Dirichlet): the couplings replace the stencil
 };
 
@@ -154,6 +156,21 @@ struct Scratch {
     void release();
 };
 
+// The word a grid's kernels report a wait that gave up in: page-locked host memory,
+// one a grid handle, so that neither another grid's solves nor another thread's
+// checks touch it.  It outlives the handle while a thread that launched solves on it
+// has not looked at it (check_gave_up).
+struct WaitFlag {
+    int* p = nullptr;
+    std::atomic<int> thread{0};  // the thread that launched the grid's last such solve
+    WaitFlag() = default;
+    WaitFlag(const WaitFlag&) = delete;
+    WaitFlag& operator=(const WaitFlag&) = delete;
+    ~WaitFlag() {
+        if (p) cudaFreeHost(p);
+    }
+};
+
 }  // namespace ew
 
 struct ew_grid {
@@ -168,6 +185,7 @@ struct ew_grid {
     ew::Scratch mgh;       // multigrid hierarchy
     ew::Scratch pairs;     // EW_FP32X2 grids: the input and output vectors as double-FP32 pairs
     ew::Scratch hostio;    // ew_filter_apply_host: device buffers of two input and two output chunks
+    std::shared_ptr<ew::WaitFlag> gave_up;  // made by the first explicit FP32 solve (geom.gave_up points to its word)
     void* host_pinned = nullptr;  // small pinned staging for reductions
     size_t host_pinned_bytes = 0;
 };
@@ -193,6 +211,11 @@ ew_status plan_filter(const GridGeom& g, const ew_filter_params* p, FilterPlan* 
 // the grid is usable on the current device (binds it on first use); bytes of one vector element
 ew_status check_grid(const ew_grid* g);
 size_t elem_size(const ew_grid* g);
+// the grid's word for waits that give up exists, and the calling thread will look at it
+ew_status arm_gave_up(ew_grid* g);
+// EW_ETIMEOUT, once, if a wait gave up in a finished solve on this grid or in one that the calling thread launched on
+// any grid; call after a synchronisation
+ew_status check_gave_up(const GridGeom& g);
 // the grid's page-locked staging buffer, at least `bytes` long
 ew_status pinned(ew_grid* g, size_t bytes, void** out);
 
@@ -234,8 +257,6 @@ const std::vector<Rb2dDesc>& rb2d_variants(int R);
 ew_status rb2d_launch(const Rb2dDesc& d, const GridGeom& g, const float* Ain, const float* Bin, float* Aout,
                       float* Bout, float* acc, const float* cw, int b, const Stencil<float>& s, int nvec,
                       int64_t fstride, cudaStream_t st);
-// reads (and clears) the flag a staging wait sets when it gives up: EW_ETIMEOUT if set
-ew_status rb2d_check_timeout();
 
 // TMA-staged persistent form of the 2D FP32 blocked step (ew_tma2d.cu)
 struct Tma2dDesc {
@@ -250,8 +271,6 @@ const std::vector<Tma2dDesc>& tma2d_variants(int R);
 ew_status tma2d_launch(const Tma2dDesc& d, const GridGeom& g, const float* Ain, const float* Bin, float* Aout,
                        float* Bout, float* acc, const float* cw, int b, const Stencil<float>& s, int nvec,
                        int64_t fstride, cudaStream_t st);
-// reads (and clears) the flag a staging wait of the TMA-staged step sets when it gives up
-ew_status tma2d_check_timeout();
 
 // the most time steps a candidate of the tuners takes in one launch: the device
 // table of filter weights holds that many entries after the solve's own
@@ -310,8 +329,6 @@ OnChipForm persist2d_form(const GridGeom& g, int nvec);
 size_t persist2d_room(const GridGeom& g, int nvec);  // bytes it needs after the time-level fields
 ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
                             int nvec, int64_t fstride, void* records, cudaStream_t st, bool* taken);
-// reads (and clears) the flag a halo exchange sets when it gives up
-ew_status persist2d_check_timeout();
 
 // --- curvilinear grids (ew_mapped.cu) ----------------------------------------
 ew_status mapped_build(int64_t n1, int64_t n2, const double* xy, MappedData* m);
@@ -325,8 +342,6 @@ ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* 
 // c the six coupling planes; accumulates into acc
 ew_status mapped_advance(const GridGeom& g, const FilterPlan& plan, const float* c, const float* cdev, float* const* F,
                          float* acc, int nvec, int64_t fstride, float dt2, cudaStream_t st);
-// reads (and clears) the flag a staging wait of the blocked curvilinear step sets when it gives up
-ew_status mapped_check_timeout();
 template <typename T>
 ew_status mapped_wsqrt(const GridGeom& g, const T* in, T* out, int nvec, int e, cudaStream_t st);
 

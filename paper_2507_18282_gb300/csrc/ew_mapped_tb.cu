@@ -31,8 +31,6 @@
 
 namespace ew {
 
-__device__ int g_mapped_timeout = 0;
-
 template <int NWX, int NTY, int KY, int B>
 struct MappedTbShape {
     static constexpr int CWX = 64 * NWX, CWY = NTY * KY;  // compute region (two columns a lane)
@@ -53,7 +51,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY, 512 / (32 * NWX * NTY))
                      const __grid_constant__ CUtensorMap mapC, int nx, int ny, int pitch,
                      const float* __restrict__ coef, float* __restrict__ Dout, float* __restrict__ Wout,
                      float* __restrict__ acc, const float* __restrict__ cw, int b, float dt2, int nvec, int vpc,
-                     int64_t fstride) {
+                     int64_t fstride, int* gave_up) {
     using S = MappedTbShape<NWX, NTY, KY, B>;
     constexpr int H = S::H, TX = S::TX, TY = S::TY, O = S::O, P = S::BOXW, BUFP = S::BUFP;
     extern __shared__ __align__(128) unsigned char smem_mt[];
@@ -112,7 +110,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY, 512 / (32 * NWX * NTY))
         if (v == v0) ok = tma_mbar_wait_bounded(&bar[0], 0u);
         ok = tma_mbar_wait_bounded(&bar[1], (unsigned)(v - v0) & 1u) && ok;
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(&g_mapped_timeout, 1);
+            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
             // no copy may outlive the CTA: give those in flight another bounded chance
             tma_mbar_wait_bounded(&bar[0], 0u);
             tma_mbar_wait_bounded(&bar[1], (unsigned)(v - v0) & 1u);
@@ -223,7 +221,7 @@ static ew_status advance(const GridGeom& g, const FilterPlan& plan, const float*
         const int b = (int)std::min<int64_t>(B, plan.Nt - L);
         cudaEvent_t ev = fused_begin(st);
         kern<<<grid, S::NT, S::SMEM, st>>>(mF[p], mF[w], mC, nx, ny, pitch, c, F[a], F[d], acc, cdev + L + 1, b, dt2,
-                                           nvec, vpc, fstride);
+                                           nvec, vpc, fstride, g.gave_up);
         EW_CUDA_TRY(cudaGetLastError());
         fused_end(ev, st, g.N * nvec, g.N * nvec * b);
         L += b;
@@ -231,14 +229,6 @@ static ew_status advance(const GridGeom& g, const FilterPlan& plan, const float*
         std::swap(w, d);
     }
     return EW_OK;
-}
-
-ew_status mapped_check_timeout() {
-    int flag = 0, zero = 0;
-    EW_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_mapped_timeout, sizeof(int)));
-    if (!flag) return EW_OK;
-    EW_CUDA_TRY(cudaMemcpyToSymbol(g_mapped_timeout, &zero, sizeof(int)));
-    return set_error(EW_ETIMEOUT, "a staging copy of the blocked curvilinear step did not complete");
 }
 
 ew_status mapped_advance(const GridGeom& g, const FilterPlan& plan, const float* c, const float* cdev, float* const* F,

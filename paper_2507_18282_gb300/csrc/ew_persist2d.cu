@@ -23,7 +23,7 @@
 //
 // The CTAs of a launch wait for one another, so the launch is cooperative (all
 // are resident, or it fails).  Every wait is bounded (about two seconds of SM
-// clock); a CTA that gives up records it in a device flag (EW_ETIMEOUT at the
+// clock); a CTA that gives up records it in the grid's flag (EW_ETIMEOUT at the
 // next synchronising call) and leaves; the others' waits run out too.
 //
 // The operations of a point and their order are those of tb2d_tile: the same
@@ -46,8 +46,6 @@
 #include "ew_tb2d_dev.cuh"
 
 namespace ew {
-
-__device__ int g_persist_timeout = 0;
 
 template <int R, int NWX, int NTY, int KY, int B>
 struct PersistShape {
@@ -76,7 +74,7 @@ template <int R, int NWX, int NTY, int KY, int B, int MINB>
 __global__ void __launch_bounds__(32 * NWX * NTY, MINB)
     k_persist2d(int nx, int ny, const float* __restrict__ Din, const float* __restrict__ Win, float* __restrict__ acc,
                 const float* __restrict__ cw, int64_t Nt, Stencil<float> st, int ntx, int nty, int64_t fstride,
-                unsigned long long* rec, int stall) {
+                unsigned long long* rec, int stall, int* gave_up) {
     using S = PersistShape<R, NWX, NTY, KY, B>;
     constexpr int RX = S::RX, RY = S::RY, PX = S::PX, OFF = S::OFF, H = S::H, NT = S::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -275,7 +273,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY, MINB)
                 }
         }
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(&g_persist_timeout, 1);
+            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
             return;
         }
         // D of the thread's points outside the tile (cells past the halo keep what they hold:
@@ -407,11 +405,13 @@ ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const flo
     int nx = (int)g.n[0], ny = (int)g.n[1], ntx = p.ntx, nty = p.nty;
     int64_t Nt = plan.Nt;
     const float *D1 = F[0], *W1 = F[1];
+    int* gave_up = g.gave_up;
     unsigned long long* rec = (unsigned long long*)records;
     int stall = getenv("EW_TEST_RB2D_STALL") ? 1 : 0;  // test hook: the first CTA publishes nothing, so the waits run out
     EW_CUDA_TRY(cudaMemsetAsync(rec, 0, persist2d_room(g, nvec), st));
     void* args[] = {(void*)&nx, (void*)&ny, (void*)&D1,  (void*)&W1,  (void*)&acc,     (void*)&cdev, (void*)&Nt,
-                    (void*)&s,  (void*)&ntx, (void*)&nty, (void*)&fstride, (void*)&rec,  (void*)&stall};
+                    (void*)&s,  (void*)&ntx, (void*)&nty, (void*)&fstride, (void*)&rec,  (void*)&stall,
+                    (void*)&gave_up};
     cudaEvent_t ev = fused_begin(st);
     cudaError_t e = getenv("EW_TEST_COOP_TOO_LARGE")  // test hook: the answer of a device with fewer SMs
                         ? cudaErrorCooperativeLaunchTooLarge
@@ -426,14 +426,6 @@ ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const flo
     EW_CUDA_TRY(e);
     fused_end(ev, st, g.N * nvec, g.N * nvec * (plan.Nt - 1));
     return EW_OK;
-}
-
-ew_status persist2d_check_timeout() {
-    int flag = 0, zero = 0;
-    EW_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_persist_timeout, sizeof(int)));
-    if (!flag) return EW_OK;
-    EW_CUDA_TRY(cudaMemcpyToSymbol(g_persist_timeout, &zero, sizeof(int)));
-    return set_error(EW_ETIMEOUT, "a halo exchange of the on-chip wave-solve did not complete");
 }
 
 }  // namespace ew

@@ -38,8 +38,6 @@
 
 namespace ew {
 
-__device__ int g_rb2d_timeout = 0;  // set when a staging wait gave up
-
 template <int R, int NTY, int KY, int B>
 struct Rb2dShape {
     static constexpr int CW = 128;        // compute-region width: 32 lanes x 4 columns
@@ -284,7 +282,7 @@ template <int R, int NTY, int KY, int B, bool GEN>
 __global__ void __launch_bounds__(32 * NTY, 1)
     k_step_rb2d(int nx, int ny, const float* __restrict__ Ain, const float* __restrict__ Bin, float* __restrict__ Aout,
                 float* __restrict__ Bout, float* __restrict__ acc, const float* __restrict__ cw, int b, Stencil<float> st,
-                int64_t fstride, int tiles_x, int tiles_per_vec, int ntiles, unsigned stall_tx) {
+                int64_t fstride, int tiles_x, int tiles_per_vec, int ntiles, unsigned stall_tx, int* gave_up) {
     using S = Rb2dShape<R, NTY, KY, B>;
     constexpr int CW = S::CW, CH = S::CH, NT = S::NT, PITCH = S::PITCH, H = S::H, TX = S::TX, TY = S::TY;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -328,7 +326,7 @@ __global__ void __launch_bounds__(32 * NTY, 1)
         const bool ok = mbar_wait_bounded(bar, phase);
         phase ^= 1u;
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(&g_rb2d_timeout, 1);
+            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
             return;
         }
         rb_fixup<CH, CW, PITCH, NT, GEN>(nx, ny, st.bc, x0, y0, stage, tid);
@@ -443,21 +441,14 @@ ew_status rb2d_launch(const Rb2dDesc& d, const GridGeom& g, const float* Ain, co
     int grid = std::min(ntiles, nsm);
     // EW_TEST_RB2D_STALL: test hook that makes every CTA's first staging wait run out
     unsigned stall_tx = getenv("EW_TEST_RB2D_STALL") ? 16u : 0u;
+    int* gave_up = g.gave_up;
     void* args[] = {(void*)&nx,   (void*)&ny, (void*)&Ain, (void*)&Bin,     (void*)&Aout,          (void*)&Bout,
                     (void*)&acc,  (void*)&cw, (void*)&b,   (void*)&s,       (void*)&fstride,       (void*)&tiles_x,
-                    (void*)&tiles_per_vec, (void*)&ntiles, (void*)&stall_tx};
+                    (void*)&tiles_per_vec, (void*)&ntiles, (void*)&stall_tx, (void*)&gave_up};
     cudaEvent_t ev = fused_begin(st);
     EW_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(d.threads), args, d.smem, st));
     fused_end(ev, st, g.N * nvec, g.N * nvec * b);
     return EW_OK;
-}
-
-ew_status rb2d_check_timeout() {
-    int flag = 0, zero = 0;
-    EW_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_rb2d_timeout, sizeof(int)));
-    if (!flag) return EW_OK;
-    EW_CUDA_TRY(cudaMemcpyToSymbol(g_rb2d_timeout, &zero, sizeof(int)));
-    return set_error(EW_ETIMEOUT, "a staging copy of the register-blocked step did not complete");
 }
 
 }  // namespace ew

@@ -64,8 +64,6 @@
 
 namespace ew {
 
-__device__ int g_tma2d_timeout = 0;
-
 template <int R, int NWX, int NTY, int KY, int B>
 struct Tma2dShape {
     static constexpr int CWX = 64 * NWX;                 // compute-region width (two columns per lane)
@@ -159,7 +157,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY + 32, 1)
                  const __grid_constant__ CUtensorMap mapAo, const __grid_constant__ CUtensorMap mapBo, int nx, int ny,
                  float* __restrict__ acc,
                  const float* __restrict__ cw, int b, Stencil<float> st, int tiles_x, int tiles_per_vec, int ntiles,
-                 unsigned stall_tx) {
+                 unsigned stall_tx, int* gave_up) {
     using S = Tma2dShape<R, NWX, NTY, KY, B>;
     constexpr int RX = S::RX, RY = S::RY, BOXW = S::BOXW, H = S::H, TX = S::TX, TY = S::TY, NTC = S::NTC,
                   BUF = S::BUF, BUFP = S::BUFP;
@@ -222,7 +220,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY + 32, 1)
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0) {
                     bulk_wait_all();
-                    atomicExch(&g_tma2d_timeout, 1);
+                    if (gave_up) *(volatile int*)gave_up = 1;
                 }
                 return;  // the compute warps give up on their next wait
             }
@@ -290,7 +288,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY + 32, 1)
         const bool ok = tma_mbar_wait_bounded(&full[s], (ph >> s) & 1u);
         ph ^= 1u << s;
         if (cbar_or<NTC>(!ok)) {
-            if (tid == 0) atomicExch(&g_tma2d_timeout, 1);
+            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
             return;  // the producer gives up on its wait for this tile
         }
         if (x0 < 0 || y0 < 0 || x0 + RX > nx || y0 + RY > ny) {
@@ -496,21 +494,14 @@ ew_status tma2d_launch(const Tma2dDesc& d, const GridGeom& g, const float* Ain, 
     int grid = std::min(ntiles, nsm);
     // EW_TEST_RB2D_STALL: test hook that makes every CTA's first staging wait run out
     unsigned stall_tx = getenv("EW_TEST_RB2D_STALL") ? 16u : 0u;
+    int* gave_up = g.gave_up;
     void* args[] = {(void*)&mA,  (void*)&mB,      (void*)&mAo,           (void*)&mBo,     (void*)&nx,
                     (void*)&ny,  (void*)&acc,     (void*)&cw,            (void*)&b,       (void*)&s,
-                    (void*)&tiles_x, (void*)&tiles_per_vec, (void*)&ntiles, (void*)&stall_tx};
+                    (void*)&tiles_x, (void*)&tiles_per_vec, (void*)&ntiles, (void*)&stall_tx, (void*)&gave_up};
     cudaEvent_t ev = fused_begin(st);
     EW_CUDA_TRY(cudaLaunchKernel(fn, dim3(grid), dim3(d.threads), args, d.smem, st));
     fused_end(ev, st, g.N * nvec, g.N * nvec * b);
     return EW_OK;
-}
-
-ew_status tma2d_check_timeout() {
-    int flag = 0, zero = 0;
-    EW_CUDA_TRY(cudaMemcpyFromSymbol(&flag, g_tma2d_timeout, sizeof(int)));
-    if (!flag) return EW_OK;
-    EW_CUDA_TRY(cudaMemcpyToSymbol(g_tma2d_timeout, &zero, sizeof(int)));
-    return set_error(EW_ETIMEOUT, "a staging copy of the TMA-staged step did not complete");
 }
 
 }  // namespace ew
