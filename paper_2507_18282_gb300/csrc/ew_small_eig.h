@@ -4,6 +4,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 namespace ew {
@@ -20,6 +21,14 @@ inline void tridiagonal_eig(int n, std::vector<double>& A, std::vector<double>& 
     auto row = [&](std::vector<double>& M, int i) { return M.data() + (size_t)i * n; };
     std::vector<double> v((size_t)n * n, 0.0), beta(n, 0.0), p(n), e(n, 0.0);
     w.assign(n, 0.0);
+    // where squares of the entries would leave the range: entries near 1 (an exact scaling)
+    double big = 0.0;
+    int ex = 0;
+    for (double a : A) big = std::max(big, fabs(a));
+    if (big > 0.0 && std::isfinite(big)) frexp(big, &ex);
+    if (ex > -300 && ex < 300) ex = 0;
+    if (ex)
+        for (double& a : A) a = ldexp(a, -ex);
     for (int k = 0; k + 2 < n; ++k) {  // reflection k zeroes column k below the subdiagonal
         double* vk = row(v, k);
         double ss = 0.0;
@@ -84,7 +93,7 @@ inline void tridiagonal_eig(int n, std::vector<double>& A, std::vector<double>& 
         int lo = hi - 1;
         while (lo > 0 && !negligible(lo - 1)) --lo;
         const double del = 0.5 * (w[hi - 1] - w[hi]), eh = e[hi - 1];
-        const double root = sqrt(del * del + eh * eh);
+        const double sq = sqrt(del * del + eh * eh), root = sq > 0.0 ? sq : hypot(del, eh);
         const double shift = w[hi] - eh * (eh / (del >= 0.0 ? del + root : del - root));
         double x = w[lo] - shift, z = e[lo];  // the bulge starts here and is chased to hi
         for (int k = lo; k < hi; ++k) {
@@ -108,6 +117,8 @@ inline void tridiagonal_eig(int n, std::vector<double>& A, std::vector<double>& 
         }
     }
     transpose();
+    if (ex)
+        for (double& a : w) a = ldexp(a, ex);
 }
 
 }  // namespace ew
