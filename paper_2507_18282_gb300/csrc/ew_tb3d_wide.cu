@@ -38,6 +38,7 @@
 // step a launch) -> 8.0 ms; 255^3 order 4 100 -> 200 Gcell-steps/s.
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <algorithm>
 #include <map>
@@ -428,6 +429,20 @@ static ew_status launch_variant(int v, int b, const GridGeom& g, const float* Di
     return launch_depth(b, g, Din, Win, Dout, Wout, acc, cw, s, nvec, fstride, st);
 }
 
+// EW_TB3D_VARIANT=wide:d or narrow:d (d = 2, 3, 4) fixes the second-order variant
+// instead of timing them, the 64 x 32 or the 32 x 32 regions at depth d: a tuning
+// and testing override.  0: not set; EW_EINVAL for any other text
+static ew_status forced_variant(int* v) {
+    *v = 0;
+    const char* e = getenv("EW_TB3D_VARIANT");
+    if (!e) return EW_OK;
+    const bool narrow = !strncmp(e, "narrow:", 7);
+    const char* d = narrow ? e + 7 : !strncmp(e, "wide:", 5) ? e + 5 : "";
+    if (d[0] < '2' || d[0] > '4' || d[1]) return set_error(EW_EINVAL, "EW_TB3D_VARIANT: wide:d or narrow:d, d = 2, 3, 4");
+    *v = (narrow ? kNarrow : 0) + d[0] - '0';
+    return EW_OK;
+}
+
 // depth autotuner (second order): times depths 2..4 on the caller's buffers
 // (before the real wave-solve overwrites them) and caches the fastest per grid
 // shape.  Fourth order: depth 2 (a rim of 4; depth 3 would leave 20 of 32 rows)
@@ -438,7 +453,9 @@ static std::mutex g_tb3w_mu;
 ew_status tb3d_wide_tune(const GridGeom& g, const FilterPlan& plan, const float* cdev, float* const* F, float* acc,
                          int nvec, int64_t fstride, cudaStream_t st) {
     if (g.order != 2) return EW_OK;
-    int dev = 0;
+    int dev = 0, forced = 0;
+    EW_TRY(forced_variant(&forced));
+    if (forced) return EW_OK;
     EW_CUDA_TRY(cudaGetDevice(&dev));
     Tb3dKey key{g.n[0], g.n[1], g.n[2], nvec, dev};
     {
@@ -486,11 +503,15 @@ ew_status tb3d_wide_advance(const GridGeom& g, const FilterPlan& plan, const flo
     if (tb > 1) {
         B = std::min(tb, B);
     } else if (g.order == 2) {
-        int dev = 0;
+        int dev = 0, forced = 0;
         EW_CUDA_TRY(cudaGetDevice(&dev));
+        EW_TRY(forced_variant(&forced));
         std::lock_guard<std::mutex> lk(g_tb3w_mu);
         auto it = g_tb3w_cache.find(Tb3dKey{g.n[0], g.n[1], g.n[2], nvec, dev});
-        if (it != g_tb3w_cache.end()) B = it->second;
+        if (forced)
+            B = forced;
+        else if (it != g_tb3w_cache.end())
+            B = it->second;
     }
     int v = 0;  // variant: below kNarrow the 64 x 32 regions
     if (B >= kNarrow) {
