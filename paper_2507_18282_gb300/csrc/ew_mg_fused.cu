@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(256)
     xc[(int64_t)J * cx + I] = T(0);
 }
 
-// partial sums of |b - M x|^2 (the
-// stopping test of a solve: no residual field is written or read back)
+// partial sums of |b - M x|^2 (the stopping test of a solve: no residual field is
+// written or read back)
 template <typename T, int ORDER>
 __global__ void __launch_bounds__(256)
     k_mg_resid_norm2d(int nx, int ny, const T* __restrict__ x, const T* __restrict__ b, Stencil<T> sa,

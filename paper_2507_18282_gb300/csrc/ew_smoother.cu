@@ -120,7 +120,10 @@ __global__ void __launch_bounds__(kThreads)
 // Sums: the running sum is a pair (hi, lo) of FP32 numbers, lo collecting the
 // rounding error of each fused multiply-add (t = fma(a, b, hi), its error
 // fma(a, b, hi - t)), four FP32 operations a term; the threads' pairs are
-// summed in FP64 in a fixed order.  Bound: FP32 pipe, 8 channels x 2 layers x
+// summed in FP64 in a fixed order.  Against exact sums of 64 threads' 4500 terms
+// each the error is 1.8e-11 of sum |a b|, that of FP32 products summed in FP64
+// 5.2e-11 (the pair keeps the products unrounded); a thread's sum must stay within
+// FP32's range, as the products had to before.  Bound: FP32 pipe, 8 channels x 2 layers x
 // 135 operations a point.  Accumulating each of the 432 terms of a point in
 // FP64 from shared memory (one thread per weight over an 8^3 tile) took
 // 3461 us on 127^3 and its serial sum over the tiles 456 us; this form and its
@@ -130,7 +133,7 @@ constexpr int kBwP = kBwX + 2;                        // row pitch: rows y .. y 
 constexpr int kBwPlane = kBwP * (kBwY + 2);
 constexpr int kBwCells = kBwPlane * (kBwZ + 2);       // tile with a halo of one
 constexpr int kBwThreads = 128;                       // warps 0, 1: dW1; warps 2, 3: dW2
-constexpr int kBwCtas = 3;                            // CTAs a SM (168 registers a thread)
+constexpr int kBwCtas = 3;                            // CTAs a SM (168 registers a thread, 72 bytes of it spilled)
 
 // one layer's sums over the rows of a staged tile (nxt columns; this thread's
 // row y of each plane z < nzt)

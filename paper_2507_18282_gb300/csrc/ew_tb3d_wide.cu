@@ -10,7 +10,7 @@
 // columns and two rows a thread, paired FP32 instructions), the box's z extent
 // is cut into chunks where the columns alone would not fill the SMs evenly,
 // and the inputs arrive ahead of their use: W^n by asynchronous copies three
-// (order 4: two) planes ahead, straight into the ring that level 1 reads its
+// planes ahead, straight into the ring that level 1 reads its
 // x/y neighbours from; D^n and the filter sums are loaded one plane ahead into
 // registers.  Each thread keeps the 2R+1 planes of its own points per level, and
 // the D of the last R planes of each level but the last, in registers; the x/y
@@ -58,10 +58,7 @@ struct Tb3wShape {
     static constexpr int H = R * B;                   // planes of lead-in and run-out, rim rows
     static constexpr int HX = (H + 1) & ~1;           // rim columns: even, so column pairs stay aligned
     static constexpr int TX = kWX - 2 * HX, TY = kWY - 2 * H;
-    #ifndef EW_PF
-#define EW_PF 3
-#endif
-    static constexpr int PF = EW_PF;                      // planes of W^n in flight
+    static constexpr int PF = 3;                      // planes of W^n in flight
     static constexpr int NW = R + 1 + PF;             // W^n ring
     static constexpr int NL = R + 1;                  // ring of each level but the last
     static constexpr size_t SMEM = sizeof(float) * (size_t)kWPlane * (NW + (B - 1) * NL);
@@ -215,12 +212,11 @@ __global__ void __launch_bounds__(kWThreads, 1)
     load_d(false, zlo - R, dnx);
     load_a(false, zlo - LA, anx);
     int ws = 0, ls = 0;  // ring slots of step z: W^n, levels
-    // the queues rotate with the step (the loop is unrolled by their length) where the filter-sum
-    // queue can rotate with them or is absent; else they are shifted
+    // the queues of W rotate with the step (the loop is unrolled by their length) where the
+    // filter-sum queue can rotate with them or is absent; else they are shifted
     constexpr bool turn = R == 2 || NA == Q;
     constexpr int U = turn ? Q : 1;
     constexpr bool rot = turn && NA == Q;
-    // the filter-sum queue rotates with the step, or is shifted
     // one plane; t = (z - zlo) mod Q: queue entry q is register (q + t + 1) mod Q
     auto step = [&](bool fast, int t, int z) {
         cp_async_wait_group<PF - 1>();  // this thread's copies of plane z have landed
@@ -328,7 +324,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
                     else
                         a = Aq[ae][j];
                     if (own[j] && (fast || z >= zs + H)) {
-                                                const int64_t at = (z - H) * plane + (o + (unsigned)(j * nx));
+                        const int64_t at = (z - H) * plane + (o + (unsigned)(j * nx));
                         Wout[at] = w.x;
                         Dout[at] = d.x;
                         acc[at] = a.x;
