@@ -593,6 +593,8 @@ static ew_status power_t(ew_grid* g, const ew_filter_params* p, T* v, int iters,
     int k = 0;
     for (k = 0; k < iters;) {
         EW_TRY(filter_apply_t<T>(g, p, plan, v, w, 1, st));      // w = S v
+        EW_TRY(pinned(g, sizeof(double) * 8, &hp));               // its weight table may have moved the staging buffer
+        h = (double*)hp;
         EW_TRY(launch_dots<T>(w, v, N, 1, dpart, dsc + 2, st));   // beta = (S v, v)
         EW_TRY(launch_dots<T>(w, w, N, 1, dpart, dsc, st));
         EW_CUDA_TRY(cudaMemcpyAsync(h, dsc, sizeof(double) * 3, cudaMemcpyDeviceToHost, st));
