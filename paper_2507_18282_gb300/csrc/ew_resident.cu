@@ -419,10 +419,14 @@ static int clusters_at_a_time(const ResidentPlan& p) {
 // narrow grids (28 columns and fewer) and more than 9500 points stay with the
 // clusters (18 x 508, 140 vectors: 306 against 258 us).  Pairs in clusters of two:
 // only a second wave of a few CTAs loses (264 x 17, 77 vectors, order 2: 269 against
-// 282 us).
+// 282 us).  FP64 is bound by the SMs' FP64 units, so two CTAs a vector gain only
+// where one CTA leaves most of a second wave empty (75 x 74, order 4, 40 steps: 228
+// vectors 1602 in clusters against 1803 us; 120 vectors of 47 x 88 839 against 699
+// us; 304 of 407 x 12, order 2, 1234 against 1049 us).
 template <typename T>
 static bool one_cta_wins(const GridGeom& g, int nvec, int C) {
     if (nvec <= 76) return false;
+    if (std::is_same<T, double>::value) return (nvec * C + 151) / 152 > (nvec + 151) / 152 * 1.6;
     if (std::is_same<T, dd>::value) return C == 2 && nvec * C > 152 && nvec * C <= 172;
     if (sizeof(T) != 4 || C != 4 || (g.order == 4 && (g.n[0] < 32 || g.N > 9500))) return false;
     return (nvec * C + 151) / 152 > (nvec + 151) / 152 * (2.6 + 1.35e-4 * (double)g.N);
