@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(kT3* kT3, 1)
 // the rows above and below as pairs.  The operations of a level and their
 // order are those of the scalar kernel above, so both give the same values.
 // The 64 x 32 regions of ew_tb3d_wide.cu are faster on large boxes (511^3 39.2
-// against 44.7 ms) but leave a narrow box's lanes idle: 27 x 463 x 132, 6 vectors,
-// 3.8 ms against 3.0 ms here; the tuner there times both.
+// against 44.7 ms) but leave a narrow box's lanes idle: 27 x 463 x 132, 6 vectors, 46
+// steps 2.49 ms against 2.06 ms here; the tuner there times both.
 template <int B, bool FULL>
 __global__ void __launch_bounds__(kT3* kT3 / 2, 1)
     k_step_tb3d_f2(int nx, int ny, int nz, const float* __restrict__ Din, const float* __restrict__ Win,

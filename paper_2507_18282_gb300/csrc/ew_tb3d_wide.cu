@@ -391,8 +391,14 @@ static ew_status launch_wide(const GridGeom& g, const float* Din, const float* W
     return EW_OK;
 }
 
-// planes are addressed with 32-bit offsets
+// Planes are addressed with 32-bit offsets.  Fourth order: a launch of two steps leads
+// in over four planes, so one vector of a few planes goes to the one-step kernel
+// (40 steps: 5^3 259 against 345 us here, 200 x 200 x 6 341 against 390, 800 x 600 x 6
+// 1009 against 1472; from eight planes on this form wins, 200 x 200 x 8 390 against 422,
+// and with several vectors, which it takes in one launch, 200 x 200 x 6, 4 vectors 560
+// against 1393).
 bool tb3d_wide_fits(const GridGeom& g, int nvec) {
+    if (g.order == 4 && nvec == 1 && g.n[2] < 8) return false;
     return g.dim == 3 && g.n[0] * g.n[1] < INT32_MAX && g.n[1] <= 65535 * 20 && nvec <= 65535;
 }
 
@@ -409,8 +415,9 @@ static ew_status launch_depth(int b, const GridGeom& g, const float* Din, const 
 }
 
 // Second order, kNarrow + depth: the 32 x 32 regions of ew_tb3d.cu.  They can win
-// where the 64 x 32 regions overhang the box by a fifth or more or the planes are
-// few (27 x 463 x 132 3.0 against 3.8 ms, 374 x 122 x 30 374 against 390 us), so
+// where the 64 x 32 regions overhang the box by a fifth or more (27 x 463 x 132, 6
+// vectors, 46 steps: 2.06 ms at depth 2 against 2.49 ms at the best depth of the wide
+// ones) or the planes are few (not always: 374 x 122 x 30 455 against 366 us), so
 // there the tuner times them too; without the tuner (a depth asked for) they take
 // the boxes up to 32 points wide.
 constexpr int kNarrow = 16;
