@@ -275,8 +275,14 @@ __global__ void __launch_bounds__(128) k_mapped_step(int nx, int ny, const T* __
     acc[v * N + q] += cn * wn;
 }
 
+// Threads of a row's blocks: whole warps of a narrow row, 128 at most.  Blocks of 128 for every row leave most of an
+// SM's warps idle on narrow grids and made the coupling planes cost what records of a point did not (FP64, 20 x 3000, 4
+// vectors, a whole solve: 412 us with records, 472 us with planes, 409 us with planes and one warp a row;
+// 63 x 2047, one vector 273, 272 and 211 us).
+static int mthreads(const GridGeom& g) { return (int)std::min<int64_t>(128, (g.n[0] + 31) / 32 * 32); }
 static dim3 mgrid(const GridGeom& g, int nvec) {
-    return dim3((unsigned)((g.n[0] + 127) / 128), (unsigned)g.n[1], (unsigned)nvec);
+    const int t = mthreads(g);
+    return dim3((unsigned)((g.n[0] + t - 1) / t), (unsigned)g.n[1], (unsigned)nvec);
 }
 
 static ew_status mapped_check(const GridGeom& g, int nvec) {
@@ -289,7 +295,7 @@ ew_status mapped_apply_L(const GridGeom& g, const T* u, T* Lu, int nvec, double 
     EW_TRY(mapped_check(g, nvec));
     const T* c = nullptr;
     EW_TRY(mapped_device<T>(g, &c, nullptr));
-    k_mapped_apply<T><<<mgrid(g, nvec), 128, 0, st>>>((int)g.n[0], (int)g.n[1], u, Lu, c, (int)pitch2d(g.n[0]), T(scale));
+    k_mapped_apply<T><<<mgrid(g, nvec), mthreads(g), 0, st>>>((int)g.n[0], (int)g.n[1], u, Lu, c, (int)pitch2d(g.n[0]), T(scale));
     EW_CUDA_TRY(cudaGetLastError());
     count_launch();
     return EW_OK;
@@ -309,7 +315,7 @@ ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* 
     const int nx = (int)g.n[0], ny = (int)g.n[1], pitch = (int)pitch2d(g.n[0]);
     const dim3 grid = mgrid(g, nvec);
     constexpr bool blocked = sizeof(T) == 4;
-    k_mapped_first<T><<<grid, 128, 0, st>>>(nx, ny, vin, F[0], F[1], vout, c, pitch, T(0.5 * plan.dt * plan.dt),
+    k_mapped_first<T><<<grid, mthreads(g), 0, st>>>(nx, ny, vin, F[0], F[1], vout, c, pitch, T(0.5 * plan.dt * plan.dt),
                                             T(plan.cn(0)), T(plan.cn(1)), fstride, blocked ? pitch : nx);
     EW_CUDA_TRY(cudaGetLastError());
     count_launch();
@@ -320,7 +326,7 @@ ew_status mapped_wave_solve(const GridGeom& g, const FilterPlan& plan, const T* 
         int cur = 1, nxt = 2;
         for (int64_t L = 1; L < plan.Nt; ++L) {
             cudaEvent_t ev = fused_begin(st);
-            k_mapped_step<T><<<grid, 128, 0, st>>>(nx, ny, F[cur], F[0], F[nxt], vout, c, pitch, dt2,
+            k_mapped_step<T><<<grid, mthreads(g), 0, st>>>(nx, ny, F[cur], F[0], F[nxt], vout, c, pitch, dt2,
                                                    T(plan.cn(L + 1)), fstride);
             EW_CUDA_TRY(cudaGetLastError());
             fused_end(ev, st, g.N * nvec, g.N * nvec);
