@@ -545,7 +545,7 @@ struct MGSolver {
     // prolongation of the coarse iterate when `correct`
     ew_status smooth2d(int L, int steps, bool correct) {
         const Stencil<T> sa = make_stencil<T>(lv[L], a);
-        const int most = mg_smooth2d_sweeps<T>(lv[L].order, p->red_black != 0);
+        const int most = mg_smooth2d_sweeps<T>(lv[L], p->red_black != 0);
         while (steps > 0) {
             const int ns = std::min(steps, most);
             EW_TRY(mg_smooth2d<T>(lv[L], X[L], B[L], Tm[L], sa, weight(L, sa), p->red_black != 0, ns,

@@ -45,7 +45,7 @@ template <typename T>
 size_t mg_bottom_smem(const int64_t* n, int nlev);
 // sweeps one launch of mg_smooth2d can take (and must be given at most)
 template <typename T>
-int mg_smooth2d_sweeps(int order, bool gs);
+int mg_smooth2d_sweeps(const GridGeom& g, bool gs);
 // xo = `sweeps` smoothing sweeps from x (+ P ec, when ec is given, ec on grid c)
 template <typename T>
 ew_status mg_smooth2d(const GridGeom& g, const T* x, const T* b, T* xo, const Stencil<T>& sa, T wd, bool gs, int sweeps,

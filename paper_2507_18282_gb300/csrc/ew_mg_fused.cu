@@ -481,12 +481,17 @@ static ew_status smooth2d_ns(const GridGeom& g, const T* x, const T* b, T* xo, c
     return smooth2d_tile<T, ORDER, GS, NS, 16>(g, x, b, xo, sa, wd, ec, c, st);
 }
 
+// Two sweeps a launch but for the three colours of reach two (one sweep already has a
+// halo of six) and the largest FP64 levels of order-4 Jacobi, whose halo points cost
+// the FP64 units more than a launch (V(2,2), four cycles: 2047^2 5042 us with two, 4830
+// with one; 1023^2 1847 and 1901)
 template <typename T>
-int mg_smooth2d_sweeps(int order, bool gs) {
-    return gs && order == 4 ? 1 : 2;  // three colours of reach two: one sweep already has a halo of six
+int mg_smooth2d_sweeps(const GridGeom& g, bool gs) {
+    if (g.order == 4) return gs || (sizeof(T) == 8 && g.N > (int64_t)2 << 20) ? 1 : 2;
+    return 2;
 }
-template int mg_smooth2d_sweeps<float>(int, bool);
-template int mg_smooth2d_sweeps<double>(int, bool);
+template int mg_smooth2d_sweeps<float>(const GridGeom&, bool);
+template int mg_smooth2d_sweeps<double>(const GridGeom&, bool);
 
 template <typename T>
 ew_status mg_smooth2d(const GridGeom& g, const T* x, const T* b, T* xo, const Stencil<T>& sa, T wd, bool gs, int sweeps,
