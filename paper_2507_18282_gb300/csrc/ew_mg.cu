@@ -28,7 +28,7 @@
 // Kernels: 3D levels run their stencil operations 2.5D blocked
 // (k_mg_plane3d), 2D levels several sweeps a launch on tiles, and the smallest
 // levels together in one launch (ew_mg_fused.cu).  1023^2 order 2 in FP64,
-// red-black, 87 cycles of a wave-solve: 58.9 -> 24.2 ms (8044 launches -> 1606).
+// red-black, 87 cycles of a wave-solve: 58.9 -> 28.6 ms (8044 launches -> 1606).
 #include <math.h>
 #include <stdlib.h>
 
@@ -559,7 +559,7 @@ struct MGSolver {
 
     // The levels from L down to the coarsest and back in one launch of one CTA,
     // once they are small: up to 31^2 points in FP64 (63^2 would take that SM's
-    // FP64 units 37 us, three launches 15-20 us), 4096 in FP32
+    // FP64 units over 37 us, three launches 15-20 us), 4096 in FP32
     bool bottom_fits(int L) const {
         if (L < p->learned_levels || L == 0 || nlev - L > kMgBottomLevels) return false;
         if (lv[L].N > (sizeof(T) == 8 ? 1024 : 4096)) return false;

@@ -10,8 +10,8 @@
 // as in ew_tb2d_dev.cuh, takes three reads and a write of it a point and step:
 // 70 % of the shared-memory bandwidth of the whole launch, and the arithmetic
 // waits for it.  Here a point takes a quarter of that: 20.5 -> 16.0 ms for 64 boxes
-// at order 2.)  What bounds it now is latency: 37 % of the paired arithmetic's
-// rate, three or four warps a scheduler, each row's chain of shuffle and seven
+// at order 2.)  What bounds it now is latency: instructions issue on 36 % of the
+// cycles, three warps a scheduler, each row's chain of shuffle and seven
 // dependent operations.  Tried: 16 warps of 6 rows 16.4 ms, 8 warps of 13 rows 17
 // ms, 20 and 24 warps spill; an mbarrier with the edge rows computed first in place
 // of the barrier 16.5 ms; descriptors fetched two tiles ahead 16.4 ms.

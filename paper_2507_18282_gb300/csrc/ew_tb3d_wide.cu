@@ -32,7 +32,7 @@
 // inputs and results move as single elements: the same kernel with 8-byte
 // copies, pair loads and pair stores on padded rows took 4.33 ms where this
 // one takes 3.55 ms (255^3, order 4, 43 steps).  Bound: instruction latency at
-// 16 warps an SM (330 instructions a warp and plane, issued on 47 % of the
+// 16 warps an SM (330 instructions a warp and plane at order 4, issued on 44 % of the
 // cycles).  Measured: 511^3 order 2, 117 steps 44.7 (32 x 32 region, one row a
 // thread) -> 39.2 ms; 191 x 161 x 143 order 4, 2 vectors, 151 steps 14.5 (one
 // step a launch) -> 8.0 ms; 255^3 order 4 100 -> 200 Gcell-steps/s.
