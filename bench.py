@@ -977,7 +977,7 @@ def run_extra(args):
         line = dict(workload="mapped2d_2047x2047_warped_square_order2_fp32_explicit", metric=METRIC, unit=UNIT,
                     value=cells / (ms / 1e3) / 1e9, ms_per_step=ms / args.steps, time_steps_per_step=info["Nt"],
                     steps_per_period=info["steps_per_period"],
-                    roofline=dict(bound="hbm", kernel="k_mapped_step<float>", bytes_per_launch=bytes_launch,
+                    roofline=dict(bound="hbm", kernel="k_step_mapped_tb", bytes_per_launch=bytes_launch,
                                   achieved=bytes_launch / (mean / 1e3) / 1e9, peak=pk["hbm_gbs"], unit="GB/s",
                                   frac=bytes_launch / (mean / 1e3) / 1e9 / pk["hbm_gbs"], peak_source=pk_kind,
                                   mean_launch_ms=mean))

@@ -433,13 +433,13 @@ static bool one_cta_wins(const GridGeom& g, int nvec, int C) {
 }
 
 // Pairs at order 4 where the clusters take several waves: a wave takes 1.4 + 0.8e-3
-// pts us a step (pts: points a CTA), the blocked kernels 9.2 us up to about 664,000
+// pts us a step (pts: points a CTA), the blocked kernels 9.2 us up to about 720,000
 // points of all vectors where their tiles fill (444 x 91, 40 steps: 14 vectors, two
 // waves, 297 against 367 us; 15 vectors, three waves, 425 against 374 us; but 59 x
 // 593, 16 vectors, 282 against 569 us)
 static bool pairs_blocked_wins(const GridGeom& g, int nvec, const ResidentPlan& p, int at_a_time) {
     const int waves = (nvec + at_a_time - 1) / at_a_time;
-    return g.order == 4 && waves > 1 && g.N * nvec <= 664000 && p.pts >= 2550 && g.n[0] >= 100 &&
+    return g.order == 4 && waves > 1 && g.N * nvec <= 720000 && p.pts >= 2550 && g.n[0] >= 100 &&
            waves * (1.4 + 0.8e-3 * p.pts) > 9.2;
 }
 
