@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY, 512 / (32 * NWX * NTY))
         if (v == v0) ok = tma_mbar_wait_bounded(&bar[0], 0u);
         ok = tma_mbar_wait_bounded(&bar[1], (unsigned)(v - v0) & 1u) && ok;
         if (__syncthreads_or(!ok)) {
-            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
+            if (tid == 0) *(volatile int*)gave_up = 1;
             // no copy may outlive the CTA: give those in flight another bounded chance
             tma_mbar_wait_bounded(&bar[0], 0u);
             tma_mbar_wait_bounded(&bar[1], (unsigned)(v - v0) & 1u);
@@ -239,6 +239,7 @@ ew_status mapped_advance(const GridGeom& g, const FilterPlan& plan, const float*
     // smaller and the depth-5 tile's (56 x 56) fewer halo points win (2047^2, 4 vectors, 1000 steps:
     // 42.8 against 46.1 ms; 1 vector: 14.3 against 13.7 ms).  Depth 3 and a 128 x 64 region a CTA of
     // 16 warps (one CTA an SM, nothing to overlap its copies with) were slower at every size.
+    if (!g.gave_up) return set_error(EW_EINVAL, "blocked curvilinear step: the grid has no word for waits that give up");
     using S5 = MappedTbShape<1, 8, 8, 5>;
     int dev = 0, nsm = 0;
     EW_CUDA_TRY(cudaGetDevice(&dev));

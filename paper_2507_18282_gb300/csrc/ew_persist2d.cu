@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY, MINB)
                 }
         }
         if (__syncthreads_or(!ok)) {
-            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
+            if (tid == 0) *(volatile int*)gave_up = 1;
             return;
         }
         // D of the thread's points outside the tile (cells past the halo keep what they hold:
@@ -408,6 +408,7 @@ ew_status persist2d_advance(const GridGeom& g, const FilterPlan& plan, const flo
     int nx = (int)g.n[0], ny = (int)g.n[1], ntx = p.ntx, nty = p.nty;
     int64_t Nt = plan.Nt;
     const float *D1 = F[0], *W1 = F[1];
+    if (!g.gave_up) return set_error(EW_EINVAL, "on-chip wave-solve: the grid has no word for waits that give up");
     int* gave_up = g.gave_up;
     unsigned long long* rec = (unsigned long long*)records;
     int stall = getenv("EW_TEST_RB2D_STALL") ? 1 : 0;  // test hook: the first CTA publishes nothing, so the waits run out

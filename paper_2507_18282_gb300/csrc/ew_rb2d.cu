@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(32 * NTY, 1)
         const bool ok = mbar_wait_bounded(bar, phase);
         phase ^= 1u;
         if (__syncthreads_or(!ok)) {
-            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
+            if (tid == 0) *(volatile int*)gave_up = 1;
             return;
         }
         rb_fixup<CH, CW, PITCH, NT, GEN>(nx, ny, st.bc, x0, y0, stage, tid);
@@ -441,6 +441,7 @@ ew_status rb2d_launch(const Rb2dDesc& d, const GridGeom& g, const float* Ain, co
     int grid = std::min(ntiles, nsm);
     // EW_TEST_RB2D_STALL: test hook that makes every CTA's first staging wait run out
     unsigned stall_tx = getenv("EW_TEST_RB2D_STALL") ? 16u : 0u;
+    if (!g.gave_up) return set_error(EW_EINVAL, "register-blocked step: the grid has no word for waits that give up");
     int* gave_up = g.gave_up;
     void* args[] = {(void*)&nx,   (void*)&ny, (void*)&Ain, (void*)&Bin,     (void*)&Aout,          (void*)&Bout,
                     (void*)&acc,  (void*)&cw, (void*)&b,   (void*)&s,       (void*)&fstride,       (void*)&tiles_x,

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY + 32, 1)
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0) {
                     bulk_wait_all();
-                    if (gave_up) *(volatile int*)gave_up = 1;
+                    *(volatile int*)gave_up = 1;
                 }
                 return;  // the compute warps give up on their next wait
             }
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(32 * NWX * NTY + 32, 1)
         const bool ok = tma_mbar_wait_bounded(&full[s], (ph >> s) & 1u);
         ph ^= 1u << s;
         if (cbar_or<NTC>(!ok)) {
-            if (tid == 0 && gave_up) *(volatile int*)gave_up = 1;
+            if (tid == 0) *(volatile int*)gave_up = 1;
             return;  // the producer gives up on its wait for this tile
         }
         if (x0 < 0 || y0 < 0 || x0 + RX > nx || y0 + RY > ny) {
@@ -494,6 +494,7 @@ ew_status tma2d_launch(const Tma2dDesc& d, const GridGeom& g, const float* Ain, 
     int grid = std::min(ntiles, nsm);
     // EW_TEST_RB2D_STALL: test hook that makes every CTA's first staging wait run out
     unsigned stall_tx = getenv("EW_TEST_RB2D_STALL") ? 16u : 0u;
+    if (!g.gave_up) return set_error(EW_EINVAL, "TMA-staged step: the grid has no word for waits that give up");
     int* gave_up = g.gave_up;
     void* args[] = {(void*)&mA,  (void*)&mB,      (void*)&mAo,           (void*)&mBo,     (void*)&nx,
                     (void*)&ny,  (void*)&acc,     (void*)&cw,            (void*)&b,       (void*)&s,
